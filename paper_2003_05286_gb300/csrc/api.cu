@@ -86,6 +86,9 @@ struct dqmc_handle_s {
   // cap on the device bytes all of the above may hold together (0: none);
   // growth past it fails with DQMC_ERR_NOMEM before any buffer is released
   size_t mem_limit = 0;
+  // set while a call that found no room for the digits of tensor-core FP64
+  // products runs without them
+  bool no_tc = false;
 };
 
 namespace {
@@ -147,6 +150,27 @@ dqmc_status ensure_ws(dqmc_handle h, size_t bytes) {
   return DQMC_OK;
 }
 
+// Sizes the workspace by layout(arena) and lays it out.  tc (whether the layout
+// holds digits of tensor-core products) is dropped when there is no room for
+// them: the call then runs those products on the FP64 pipe.
+template <class F>
+dqmc_status place(dqmc_handle h, bool& tc, F&& layout) {
+  Arena measure;
+  layout(measure);
+  dqmc_status rc = ensure_ws(h, measure.off);
+  if (rc == DQMC_ERR_NOMEM && tc && !h->capturing) {
+    tc = false;
+    Arena again;
+    layout(again);
+    rc = ensure_ws(h, again.off);
+  }
+  if (rc != DQMC_OK) return rc;
+  Arena ar;
+  ar.base = h->ws;
+  layout(ar);
+  return DQMC_OK;
+}
+
 cudaEvent_t pool_event(dqmc_handle h) {
   if (!h->pool.empty()) {
     cudaEvent_t e = h->pool.back();
@@ -192,6 +216,7 @@ unsigned long long check_word_lu(bool clear);
 unsigned long long check_word_jacobi(bool clear);
 unsigned long long check_word_chain_small(bool clear);
 unsigned long long check_word_ozaki(bool clear);
+unsigned long long check_word_gemm_tc(bool clear);
 }  // namespace dqmc
 namespace {
 struct CheckUnit {
@@ -202,7 +227,7 @@ const CheckUnit kCheckUnits[] = {
     {"api.cu", dqmc::check_word_api},         {"gemm_f64.cu", dqmc::check_word_gemm},
     {"qrp_f64.cu", dqmc::check_word_qrp},     {"lu_f64.cu", dqmc::check_word_lu},
     {"jacobi_f64.cu", dqmc::check_word_jacobi}, {"chain_small.cu", dqmc::check_word_chain_small},
-    {"ozaki_tc.cu", dqmc::check_word_ozaki},
+    {"ozaki_tc.cu", dqmc::check_word_ozaki}, {"gemm_tc.cu", dqmc::check_word_gemm_tc},
 };
 #endif
 
@@ -338,6 +363,125 @@ struct Slots {
   double* X2 = nullptr;
 };
 
+inline int pad_to(int n, int m) { return (n + m - 1) / m * m; }
+
+// Digits of the operands of tensor-core FP64 products (gemm_tc.cu) for up to
+// `cap` instances at a time; off (cap 0): the products run on the FP64 pipe.
+struct TcWs {
+  int cap = 0;
+  __nv_bfloat16 *A = nullptr, *B = nullptr;   // per-instance operands
+  int *eA = nullptr, *eB = nullptr;
+  __nv_bfloat16 *Es = nullptr;                // an operand shared by all instances
+  int* eEs = nullptr;
+};
+
+// Which FP64 products take the tensor cores, by N alone so that an instance's
+// result does not depend on its batch.  A product there is one or two splits
+// and one launch of padded 128 x 64 tiles with about 10 us of fixed cost (TMEM
+// allocation, copies, epilogue).  Equal-time chain, 64 instances, M = 50, FP64
+// pipe -> tensor cores: N = 48 3.3 -> 4.1 ms, N = 64 5.7 -> 5.2, N = 81 12.3 ->
+// 7.2, N = 100 14.2 -> 9.3.  The tree fold has few instances and small level
+// products: one instance, M = 100, N = 64 3.71 -> 3.97 ms, N = 81 5.66 -> 5.67,
+// N = 121 11.3 -> 11.1, N = 256 61.4 -> 55.2.
+constexpr int TC_MIN_N = 64, TC_TREE_MIN_N = 96;
+constexpr long long TC_SCRATCH = 512LL << 20;   // bytes of digits a TcWs may hold
+constexpr int TC_SHARES = 8;                    // products side by side (kMaxJobs)
+
+inline bool tc_wanted(dqmc_handle h, int N) {
+  return !h->no_tc && N >= TC_MIN_N && N <= TC_MAX_N;
+}
+
+void take_tc(Arena& ar, long long batch, int N, TcWs& w) {
+  const long long ea = tc_plane_elems(N, 128), eb = tc_plane_elems(N, 64);
+  long long cap = TC_SCRATCH / (2 * (ea + eb));
+  cap = cap > 65535 ? 65535 : (cap < 1 ? 1 : cap);
+  batch += TC_SHARES - 1;                     // so that an equal share still holds its part
+  w.cap = (int)(batch < cap ? batch : cap);
+  w.A = ar.take<__nv_bfloat16>(w.cap * ea);
+  w.B = ar.take<__nv_bfloat16>(w.cap * eb);
+  w.eA = ar.take<int>((long long)w.cap * pad_to(N, 128));
+  w.eB = ar.take<int>((long long)w.cap * pad_to(N, 64));
+  w.Es = ar.take<__nv_bfloat16>(ea);          // either side (ea >= eb)
+  w.eEs = ar.take<int>(pad_to(N, 128));
+}
+
+// Share q of nj of the digit slots, for products that run side by side (the
+// shared operand stays common).
+TcWs tc_part(const TcWs& w, int q, int nj, int N) {
+  TcWs p = w;
+  p.cap = w.cap / nj;
+  p.A += (long long)q * p.cap * tc_plane_elems(N, 128);
+  p.B += (long long)q * p.cap * tc_plane_elems(N, 64);
+  p.eA += (long long)q * p.cap * pad_to(N, 128);
+  p.eB += (long long)q * p.cap * pad_to(N, 64);
+  return p;
+}
+
+// Left (R = 128: rows of op(X)) or right (R = 64: columns of op(X)) operand of
+// an N x N product; one instance when sX == 0.
+TcSplitArgs tc_operand(int N, int R, const double* X, long long ld, long long sX, int trans,
+                       __nv_bfloat16* S, int* e) {
+  TcSplitArgs a;
+  a.X = X; a.sX = sX;
+  // left: element (k, row) of op(X) is X[row ld + k]; right: (k, col) is X[k ld + col]
+  const bool along_k = (R == 128) != (trans != 0);
+  a.ldm = along_k ? 1 : ld;
+  a.ldj = along_k ? ld : 1;
+  a.N = N; a.R = R; a.PJ = pad_to(N, R); a.PM = pad_to(N, 32);
+  a.S = S; a.sS = tc_plane_elems(N, R);
+  a.e = e; a.se = a.PJ;
+  return a;
+}
+
+// One batched N x N product of the method: on the tensor cores when t has
+// room, else on the FP64 pipe.  shared_A / shared_B: t.Es already holds that
+// operand's digits.  A diagonal ms between the operands goes to the
+// per-instance one.
+dqmc_status product(dqmc_handle h, int cls, double flops, const GemmArgs& g, const TcWs& t,
+                    int* status, int status_div = 1, bool shared_A = false,
+                    bool shared_B = false) {
+  if (t.cap <= 0 || g.cs || g.addIdentity || g.alpha_ptr || g.skip_if || g.divA != 1 ||
+      g.divB != 1 || g.divC != 1 || (shared_A && shared_B)) {
+    CKP(cls, flops, gemm_f64(g, h->cur));
+    return DQMC_OK;
+  }
+  const int N = g.N;
+  TcSplitArgs sa = tc_operand(N, 128, g.A, g.lda, g.sA, g.transA, t.A, t.eA);
+  TcSplitArgs sb = tc_operand(N, 64, g.B, g.ldb, g.sB, g.transB, t.B, t.eB);
+  sb.gm = g.permB; sb.sgm = g.sperm;
+  TcSplitArgs& sm = shared_B ? sa : sb;
+  sm.sc = g.ms; sm.ssc = g.sms; sm.ssc_inner = g.sms_inner; sm.divS = g.divS;
+  sa.lim = sb.lim = g.lim; sa.lim_at = sb.lim_at = g.lim_at;
+  for (int b0 = 0; b0 < g.batch; b0 += t.cap) {
+    const int nb = g.batch - b0 < t.cap ? g.batch - b0 : t.cap;
+    sa.b0 = sb.b0 = b0;
+    if (!shared_A) CK(tc_split(sa, nb, h->cur));
+    if (!shared_B) CK(tc_split(sb, nb, h->cur));
+    TcGemmArgs m;
+    m.A = shared_A ? t.Es : t.A; m.eA = shared_A ? t.eEs : t.eA;
+    m.sA = shared_A ? 0 : sa.sS; m.seA = shared_A ? 0 : sa.se;
+    m.B = shared_B ? t.Es : t.B; m.eB = shared_B ? t.eEs : t.eB;
+    m.sB = shared_B ? 0 : sb.sS; m.seB = shared_B ? 0 : sb.se;
+    m.N = N; m.nkb = sa.PM / 32; m.upperA = g.upperA; m.b0 = b0;
+    m.C = g.C; m.ldc = g.ldc; m.sC = g.sC;
+    m.scaled = g.rs || g.alpha != 1.0; m.alpha = g.alpha;
+    m.rs = g.rs; m.srs = g.srs; m.divS = g.divS;
+    m.status = status; m.status_div = status_div;
+    m.lim = g.lim; m.lim_at = g.lim_at;
+    m.csrc = g.B; m.scsrc = g.sB; m.ldcsrc = g.ldb;
+    CKP(cls, flops * nb / g.batch, tc_gemm(m, nb, h->cur));
+  }
+  return DQMC_OK;
+}
+
+// Digits of a matrix all instances share, as the left or right operand.
+dqmc_status share_operand(dqmc_handle h, const double* X, int N, int R, int trans,
+                          const TcWs& t) {
+  if (t.cap <= 0) return DQMC_OK;
+  CK(tc_split(tc_operand(N, R, X, N, 0, trans, t.Es, t.eEs), 1, h->cur));
+  return DQMC_OK;
+}
+
 struct ChainWs {
   double *C0, *C1, *W, *T;
   int* perm;
@@ -349,9 +493,9 @@ struct ChainWs {
   // per-instance slices of T' for the X update on the tensor cores
   __nv_bfloat16* ozT = nullptr;
   int* ozeT = nullptr;
+  // FP64 chain on the tensor cores: digits, with E (or E^T) as the shared operand
+  TcWs tc;
 };
-
-inline int pad_to(int n, int m) { return (n + m - 1) / m * m; }
 
 // Digit slices of E (forward chain, transposeE = 0) or E^T (backward chain)
 // into a chain workspace's shared A-operand buffers.
@@ -405,7 +549,8 @@ dqmc_status chunk_products(dqmc_handle h, int dir, int batch, int N, int M, int 
   long long sprev = s.instU;
   double* bufs[2] = {w.C0, w.C1};
   int nb = 0;
-  if (w.oz_s == 0 && N <= CHAIN_SMALL_MAX_N && batch <= 65535 && (dir > 0 || !lim)) {
+  if (w.oz_s == 0 && w.tc.cap == 0 && N <= CHAIN_SMALL_MAX_N && batch <= 65535 &&
+      (dir > 0 || !lim)) {
     // small N: the whole chunk in one launch, each CTA applying every slice
     // to a block of columns held in shared memory
     ChainSmallArgs cs;
@@ -458,7 +603,7 @@ dqmc_status chunk_products(dqmc_handle h, int dir, int batch, int N, int M, int 
       g.transA = 1;                                          // diag(e^{V_l}) E^T A
       g.rs = expV + (long long)(l - 1) * N; g.srs = sV;
     }
-    CKP(PC_CHAIN, 2.0 * N * N * (double)N * batch, gemm_f64(g, st));
+    CKS(product(h, PC_CHAIN, 2.0 * N * N * (double)N * batch, g, w.tc, status, 1, true));
     prev = bufs[nb];
     sprev = NN;
     nb ^= 1;
@@ -537,7 +682,7 @@ dqmc_status chunk_xupdate(dqmc_handle h, int dir, int batch, int N, int k, int c
   g.permB = jac ? nullptr : w.perm; g.sperm = N;
   g.C = slotX(s, dst); g.ldc = N; g.sC = s.instX;
   g.lim = lim; g.lim_at = c * k + 1;
-  CKP(PC_XUPD, (double)N * N * (double)N * batch, gemm_f64(g, st));
+  CKS(product(h, PC_XUPD, (double)N * N * (double)N * batch, g, w.tc, status));
   return DQMC_OK;
 }
 
@@ -619,6 +764,7 @@ void make_sub_jobs(ChainJob* J, int nj, int dir, int batch, int N, const double*
       J[q].w.ozT += o * cw.oz_s * (long long)cw.oz_P128 * cw.oz_PK;
       J[q].w.ozeT += o * cw.oz_P128;
     }
+    J[q].w.tc = tc_part(cw.tc, q, nj, N);
     J[q].status = status + o;
     J[q].lim = lim ? lim + o : nullptr;
     o += nb;
@@ -633,7 +779,7 @@ bool pipeline_enabled() {
 
 // Number of staggered sub-batches of an equal-time chain: DQMC_PIPELINE=n
 // (2..8) overrides the default (2 for FP64 products, 4 for tensor-core ones).
-constexpr int kMaxJobs = 8;
+constexpr int kMaxJobs = TC_SHARES;
 int pipeline_jobs(bool mixed) {
   const char* e = getenv("DQMC_PIPELINE");
   if (e && e[0] >= '2' && e[0] <= '8' && e[1] == 0) return e[0] - '0';
@@ -711,6 +857,7 @@ struct TreeWs {
   double *Iden, *C0, *C1, *U[2], *D[2], *X[2], *W, *T;
   int *perm, *len;
   int P0 = 1;
+  TcWs tc;
 };
 
 int tree_width(int nc) {
@@ -757,7 +904,8 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
   double* bufs[2] = {w.C0, w.C1};
   const double* prev = w.Iden;
   long long sprev = 0;
-  const bool small = N <= CHAIN_SMALL_MAX_N && Q <= 65535;
+  const bool small = N <= CHAIN_SMALL_MAX_N && Q <= 65535 && w.tc.cap == 0;
+  CKS(share_operand(h, E, N, 128, 0, w.tc));
   if (small) {
     // small N: the k slices of every chunk in one launch (padding chunks copy
     // the identity through)
@@ -781,7 +929,7 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     g.ms = expV + (long long)i * N; g.sms = sV; g.divS = P0; g.sms_inner = (long long)k * N;
     g.lim = w.len; g.lim_at = i + 1;
     g.tile = h->gemm_tile;
-    CKP(PC_CHAIN, f2 * Q, gemm_f64(g, st));
+    CKS(product(h, PC_CHAIN, f2 * Q, g, w.tc, status, P0, true));
     prev = bufs[i & 1];
     sprev = NN;
   }
@@ -807,7 +955,7 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     g.permB = w.perm; g.sperm = N;
     g.C = w.X[0]; g.ldc = N; g.sC = NN;
     g.lim = w.len; g.lim_at = 1;
-    CKP(PC_XUPD, (double)N * N * (double)N * Q, gemm_f64(g, st));
+    CKS(product(h, PC_XUPD, (double)N * N * (double)N * Q, g, w.tc, status, P0));
   }
   // levels: pair i of instance b = (left 2i+1, right 2i) -> i
   int cur = 0;
@@ -822,7 +970,7 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     gy.rs = w.D[cur] + N; gy.srs = 2LL * N;
     gy.C = Y; gy.ldc = N; gy.sC = NN;
     gy.tile = h->gemm_tile;
-    CKP(PC_OTHER, f2 * B2, gemm_f64(gy, st));
+    CKS(product(h, PC_OTHER, f2 * B2, gy, w.tc, status, np));
     QrpArgs q;                                        // Y D_1 = u d x
     q.N = N; q.batch = B2;
     q.A = Y; q.sA = NN;
@@ -844,7 +992,7 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     gu.B = Uq; gu.ldb = N; gu.sB = NN;
     gu.C = w.U[nxt]; gu.ldc = N; gu.sC = NN;
     gu.tile = h->gemm_tile;
-    CKP(PC_OTHER, f2 * B2, gemm_f64(gu, st));
+    CKS(product(h, PC_OTHER, f2 * B2, gu, tc_part(w.tc, 0, 2, N), status, np));
     GemmArgs gx;                                      // X = x X_1
     gx.M = gx.N = gx.K = N; gx.batch = B2;
     gx.A = w.T; gx.lda = N; gx.sA = NN; gx.upperA = 1;
@@ -852,8 +1000,10 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     gx.permB = w.perm; gx.sperm = N;
     gx.C = w.X[nxt]; gx.ldc = N; gx.sC = NN;
     h->cur = sx;
-    CKP(PC_XUPD, (double)N * N * (double)N * B2, gemm_f64(gx, sx));
+    const dqmc_status rx = product(h, PC_XUPD, (double)N * N * (double)N * B2, gx,
+                                   tc_part(w.tc, 1, 2, N), status, np);
     h->cur = st;
+    CKS(rx);
     if (cudaEventRecord(join, sx) != cudaSuccess || cudaStreamWaitEvent(st, join, 0) != cudaSuccess)
       return DQMC_ERR_CUDA;
     cur = nxt;
@@ -1269,7 +1419,12 @@ static dqmc_status graph_call(dqmc_handle h, GraphKey key, F&& body) {
   if (!h->gstream && cudaStreamCreateWithFlags(&h->gstream, cudaStreamNonBlocking) != cudaSuccess)
     return DQMC_ERR_CUDA;
   cudaStream_t caller = h->stream;
-  for (int attempt = 0; attempt < 2; ++attempt) {
+  h->no_tc = false;
+  struct Restore {   // no_tc holds for this call only
+    dqmc_handle h;
+    ~Restore() { h->no_tc = false; }
+  } restore{h};
+  for (int attempt = 0; attempt < 3; ++attempt) {
     h->stream = h->gstream;
     if (cudaStreamBeginCapture(h->gstream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
       h->stream = caller;
@@ -1286,7 +1441,12 @@ static dqmc_status graph_call(dqmc_handle h, GraphKey key, F&& body) {
     if (rc == DQMC_ERR_NOMEM && h->ws_need) {   // grow outside the capture, then record again
       if (g) cudaGraphDestroy(g);
       cudaGetLastError();
-      CKS(ensure_ws(h, h->ws_need));
+      const dqmc_status grown = ensure_ws(h, h->ws_need);
+      if (grown != DQMC_OK) {
+        if (grown != DQMC_ERR_NOMEM || h->no_tc) return grown;
+        h->no_tc = true;   // record again without the digits of tensor-core products
+        continue;
+      }
       key.v[key.n - 2] = (unsigned long long)(uintptr_t)h->ws;
       continue;
     }
@@ -1345,6 +1505,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   const long long Mp = (long long)mp_chunks * k;
   TreeWs tw;
   PlainWs pw;
+  bool tc = tc_wanted(h, N) && h->prec == DQMC_CHAIN_FP64 && (!tree || N >= TC_TREE_MIN_N);
 
   auto layout = [&](Arena& ar, ExpmWs& ew, ChainWs& cw, LohWs& lw, double*& E, double*& expV,
                     double*& U, double*& D, double*& X0, double*& X1, int*& st, HostIO& io,
@@ -1354,6 +1515,8 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
     expV = ar.take<double>(Mp * N * batch);
     if (tree) {
       take_tree(ar, batch, N, nc, tw);
+      tw.tc = TcWs{};
+      if (tc) take_tc(ar, (long long)batch * tw.P0, N, tw.tc);
       U = D = X0 = X1 = nullptr;
     } else {
       U = ar.take<double>(NN * batch);
@@ -1361,6 +1524,8 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       X0 = ar.take<double>(NN * batch);
       X1 = ar.take<double>(NN * batch);
       take_chain(ar, batch, N, cw);
+      cw.tc = TcWs{};
+      if (tc) take_tc(ar, batch, N, cw.tc);
     }
     if (h->prec != DQMC_CHAIN_FP64) take_ozaki(ar, batch, N, (int)h->prec, cw);
     take_loh(ar, batch, N, lw);
@@ -1377,12 +1542,9 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   ExpmWs ew; ChainWs cw; LohWs lw; HostIO io;
   double *E, *expV, *U, *D, *X0, *X1, *Gd = nullptr, *ldd = nullptr;
   int *stat, *sgd = nullptr;
-  Arena measure;
-  layout(measure, ew, cw, lw, E, expV, U, D, X0, X1, stat, io, Gd, ldd, sgd);
-  CKS(ensure_ws(h, measure.off));
-  Arena ar;
-  ar.base = h->ws;
-  layout(ar, ew, cw, lw, E, expV, U, D, X0, X1, stat, io, Gd, ldd, sgd);
+  CKS(place(h, tc, [&](Arena& ar) {
+    layout(ar, ew, cw, lw, E, expV, U, D, X0, X1, stat, io, Gd, ldd, sgd);
+  }));
   cudaStream_t st = h->cur;
 
   const double* Kd = K;
@@ -1415,6 +1577,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
     CKS(run_inversion(h, batch, N, Ut, NN, Dt, N, Xt, NN, Gout, ldout, sgout, stout, lw, pw));
   } else {
     if (cw.oz_s > 0) CK(split_E(E, N, 0, cw, st));   // E slices, shared by all instances
+    CKS(share_operand(h, E, N, 128, 0, cw.tc));
     CK(set_identity(U, NN, N, batch, st));
     CK(set_const(D, (long long)N * batch, 1.0, st));
     CK(set_identity(X0, NN, N, batch, st));
@@ -1622,6 +1785,8 @@ dqmc_status run_stacks(dqmc_handle h, int batch, int N, int M, int k, const doub
     CK(split_E(E, N, 0, cw, st));
     CK(split_E(E, N, 1, cw2, st));
   }
+  CKS(share_operand(h, E, N, 128, 0, cw.tc));
+  CKS(share_operand(h, E, N, 128, 1, cw2.tc));
   CK(set_identity(w.UF, nt * NN, N, batch, st));
   CK(set_const_strided(w.DF, (long long)nt * N, N, batch, 1.0, st));
   CK(set_identity(w.XF, nt * NN, N, batch, st));
@@ -1670,7 +1835,7 @@ void take_mid(Arena& ar, long long Q, int N, int ncols, MidWs& w) {
 // G(tau,0) to Gt0 and G(0,tau) to G0t (each may be null), each Q x N x N.
 dqmc_status run_two_stack_inversion(dqmc_handle h, int Q, int N, int nt, const StackWs& w,
                                     const MidWs& m, double* Gtt, double* Gt0, double* G0t,
-                                    int* status) {
+                                    int* status, const TcWs& tc) {
   cudaStream_t st = h->cur;
   const long long NN = (long long)N * N;
   const bool want_z = Gtt || G0t;                      // Z = mid^{-1} a_p^{-1} U_F^T
@@ -1682,13 +1847,13 @@ dqmc_status run_two_stack_inversion(dqmc_handle h, int Q, int N, int nt, const S
   g1.A = w.UF; g1.lda = N; g1.sA = NN; g1.transA = 1;
   g1.B = w.Ub; g1.ldb = N; g1.sB = NN;
   g1.C = m.C1; g1.ldc = N; g1.sC = NN;
-  CKP(PC_OTHER, gflops, gemm_f64(g1, st));
+  CKS(product(h, PC_OTHER, gflops, g1, tc, status, nt));
   GemmArgs g2;                                         // C2 = X_F T_b^T
   g2.M = g2.N = g2.K = N; g2.batch = Q;
   g2.A = w.XF; g2.lda = N; g2.sA = NN;
   g2.B = w.Tb; g2.ldb = N; g2.sB = NN; g2.transB = 1;
   g2.C = m.C2; g2.ldc = N; g2.sC = NN;
-  CKP(PC_OTHER, gflops, gemm_f64(g2, st));
+  CKS(product(h, PC_OTHER, gflops, g2, tc, status, nt));
   Axpby2Args ax;                                       // mid
   ax.N = N; ax.batch = Q;
   ax.A = m.C1; ax.sA = NN;
@@ -1718,7 +1883,7 @@ dqmc_status run_two_stack_inversion(dqmc_handle h, int Q, int N, int nt, const S
     g.B = m.Z + ((part == 1 && want_z) ? N : 0); g.ldb = ncols; g.sB = (long long)N * ncols;
     g.ms = m.bpinv; g.sms = N;
     g.C = out; g.ldc = N; g.sC = NN;
-    CKP(PC_OTHER, gflops, gemm_f64(g, st));
+    CKS(product(h, PC_OTHER, gflops, g, tc, status, nt));
   }
   if (G0t) {
     // b_m overwrites b_p^{-1}: the products above are ahead of it on the stream
@@ -1730,7 +1895,7 @@ dqmc_status run_two_stack_inversion(dqmc_handle h, int Q, int N, int nt, const S
     g.ms = m.bpinv; g.sms = N;
     g.alpha = -1.0;
     g.C = G0t; g.ldc = N; g.sC = NN;
-    CKP(PC_OTHER, gflops, gemm_f64(g, st));
+    CKS(product(h, PC_OTHER, gflops, g, tc, status, nt));
   }
   return DQMC_OK;
 }
@@ -1929,6 +2094,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
   double *gq[3] = {nullptr, nullptr, nullptr}, *gtmp = nullptr;   // grid values (all_tau)
   int* stat;
   int* shiftd = nullptr;
+  bool tc = tc_wanted(h, N);
   auto layout = [&](Arena& ar) {
     take_expm(ar, N, ew);
     expV = ar.take<double>(Mp * N * batch);
@@ -1942,6 +2108,12 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
     }
     take_chain(ar, batch, N, cw);
     take_chain(ar, batch, N, cw2);
+    cw.tc = cw2.tc = TcWs{};
+    if (tc) {
+      // the first also serves the products over all stack slots after the chains
+      take_tc(ar, Q, N, cw.tc);
+      take_tc(ar, batch, N, cw2.tc);
+    }
     if (h->prec != DQMC_CHAIN_FP64) {
       take_ozaki(ar, batch, N, (int)h->prec, cw);
       take_ozaki(ar, batch, N, (int)h->prec, cw2);
@@ -1959,12 +2131,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       G0td = G0t ? ar.take<double>(batch * outlen) : nullptr;
     }
   };
-  Arena measure;
-  layout(measure);
-  CKS(ensure_ws(h, measure.off));
-  Arena ar;
-  ar.base = h->ws;
-  layout(ar);
+  CKS(place(h, tc, layout));
   cudaStream_t st = h->cur;
   const double* Kd = K;
   const double* Vd = V;
@@ -1991,7 +2158,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
   if (all_tau)
     for (int i = 0; i < 3; ++i) out[i] = gq[i];
   CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, out[0], plain_t0 ? nullptr : out[1],
-                              out[2], stout));
+                              out[2], stout, cw.tc));
   if (plain_t0) CKS(run_inv_sum_t0(h, (int)Q, N, nt, sw, sumw, out[1], stout));
   if (all_tau) {
     // tau between grid points: k - 1 one-slice steps from every grid value,
@@ -2002,6 +2169,11 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
     if (expmV) CK(exp_pad(Vd, expmV, batch, M, (int)Mp, N, -1.0, nullptr, st, sh));
     double* dst[3] = {Gtto, Gt0o, G0to};
     const double f2 = 2.0 * N * (double)N * N * Q;
+    // E is still the shared left operand of cw.tc; E^{-1} becomes the shared
+    // right operand in the backward chain's slot
+    CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
+    TcWs wr = cw.tc;
+    wr.Es = cw2.tc.Es; wr.eEs = cw2.tc.eEs;
     for (int s = 0; s < k; ++s) {
       for (int i = 0; i < 3; ++i)
         if (out[i]) CK(scatter_tau(out[i], Q, nt, N, k, M, s, dst[i], st));
@@ -2022,19 +2194,19 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       right.ldc = N; right.sC = NN;
       if (out[1]) {
         left.B = out[1]; left.C = gtmp;
-        CKP(PC_OTHER, f2, gemm_f64(left, st));
+        CKS(product(h, PC_OTHER, f2, left, cw.tc, stout, nt, true));
         std::swap(out[1], gtmp);
       }
       if (out[2]) {
         right.A = out[2]; right.C = gtmp;
-        CKP(PC_OTHER, f2, gemm_f64(right, st));
+        CKS(product(h, PC_OTHER, f2, right, wr, stout, nt, false, true));
         std::swap(out[2], gtmp);
       }
       if (out[0]) {
         left.B = out[0]; left.C = gtmp;
-        CKP(PC_OTHER, f2, gemm_f64(left, st));
+        CKS(product(h, PC_OTHER, f2, left, cw.tc, stout, nt, true));
         right.A = gtmp; right.C = out[0];
-        CKP(PC_OTHER, f2, gemm_f64(right, st));
+        CKS(product(h, PC_OTHER, f2, right, wr, stout, nt, false, true));
       }
     }
   }
@@ -2088,6 +2260,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
   ExpmWs ew, ewi; ChainWs cw, cw2; StackWs sw; MidWs mw; LohWs lw; HostIO io;
   double *expV, *expmV, *Gw, *W1, *dVd = nullptr, *ldd = nullptr;
   int *stat, *sgd = nullptr;
+  bool tc = tc_wanted(h, N);
   auto layout = [&](Arena& ar) {
     take_expm(ar, N, ew);
     take_expm(ar, N, ewi);
@@ -2095,6 +2268,12 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
     expmV = ar.take<double>(Mp * N * batch);
     take_chain(ar, batch, N, cw);
     take_chain(ar, batch, N, cw2);
+    cw.tc = cw2.tc = TcWs{};
+    if (tc) {
+      // the first also serves the products over all stack slots after the chains
+      take_tc(ar, Q, N, cw.tc);
+      take_tc(ar, batch, N, cw2.tc);
+    }
     if (h->prec != DQMC_CHAIN_FP64) {
       take_ozaki(ar, batch, N, (int)h->prec, cw);
       take_ozaki(ar, batch, N, (int)h->prec, cw2);
@@ -2113,12 +2292,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       sgd = ar.take<int>(batch);
     }
   };
-  Arena measure;
-  layout(measure);
-  CKS(ensure_ws(h, measure.off));
-  Arena ar;
-  ar.base = h->ws;
-  layout(ar);
+  CKS(place(h, tc, layout));
   cudaStream_t st = h->cur;
   const double* Kd = K;
   const double* Vd = V;
@@ -2143,7 +2317,10 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
   CKS(run_loh(h, batch, N, sw.UF + nc * NN, nt * NN, sw.DF + (long long)nc * N, (long long)nt * N,
               sw.XF + nc * NN, nt * NN, nullptr, ldo, sgo, stout, lw));
   // checkpoints G_{jk+1}
-  CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, Gw, nullptr, nullptr, stout));
+  CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, Gw, nullptr, nullptr, stout, cw.tc));
+  CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
+  TcWs wr = cw.tc;                                     // E^{-1} as the shared right operand
+  wr.Es = cw2.tc.Es; wr.eEs = cw2.tc.eEs;
   const double wflops = 2.0 * N * (double)N * N * Q;
   for (int s = 0; s < k; ++s) {
     CK(grad_readout(Gw, N, (int)Q, nt, k, M, s, dVo, st));
@@ -2154,14 +2331,14 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
     a.B = Gw; a.ldb = N; a.sB = NN;
     a.ms = expV + (long long)s * N; a.sms = Mp * N; a.sms_inner = (long long)k * N; a.divS = nt;
     a.C = W1; a.ldc = N; a.sC = NN;
-    CKP(PC_OTHER, wflops, gemm_f64(a, st));
+    CKS(product(h, PC_OTHER, wflops, a, cw.tc, stout, nt, true));
     GemmArgs b;                                        // G_{l+1} = W1 diag(e^{-V_l}) E^{-1}
     b.M = b.N = b.K = N; b.batch = (int)Q;
     b.A = W1; b.lda = N; b.sA = NN;
     b.B = ewi.t0; b.ldb = N; b.sB = 0;
     b.ms = expmV + (long long)s * N; b.sms = Mp * N; b.sms_inner = (long long)k * N; b.divS = nt;
     b.C = Gw; b.ldc = N; b.sC = NN;
-    CKP(PC_OTHER, wflops, gemm_f64(b, st));
+    CKS(product(h, PC_OTHER, wflops, b, wr, stout, nt, false, true));
   }
   if (host) {
     bool ok = true;
@@ -2261,6 +2438,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
   const int s_digits = mixed ? (int)h->prec : 0;
   // ---- workspace (h->ws) and index tables (h->rtab): one region per group ----
   std::vector<RaggedGroupWs> gw(groups.size());
+  bool tc = true;
   auto layout = [&](Arena& ar) {
     for (size_t i = 0; i < groups.size(); ++i) {
       const RaggedGroup& g = groups[i];
@@ -2275,6 +2453,8 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       w.X0 = ar.take<double>(NN * nb);
       w.X1 = ar.take<double>(NN * nb);
       take_chain(ar, nb, N, w.cw);
+      w.cw.tc = TcWs{};
+      if (tc && !mixed && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
       if (mixed) take_ozaki(ar, nb, N, s_digits, w.cw);
       take_loh(ar, nb, N, w.lw);
       if (h->inv == DQMC_INV_PLAIN) take_plain(ar, nb, N, w.pw);
@@ -2293,13 +2473,9 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       gw[i].offG = ar.take<long long>(nb);
     }
   };
-  Arena measure, measure_t;
-  layout(measure);
+  Arena measure_t;
   layout_tables(measure_t);
-  CKS(ensure_ws(h, measure.off));
-  Arena ar;
-  ar.base = h->ws;
-  layout(ar);
+  CKS(place(h, tc, layout));
   if (measure_t.off > h->rtab_bytes) {
     if (h->capturing) return DQMC_ERR_UNSUPPORTED;
     if (!within_limit(h, h->rtab_bytes, measure_t.off)) return DQMC_ERR_NOMEM;
@@ -2387,6 +2563,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
         if (!E_pool) CKS(run_expm(h, K_pool + g.offK, N, g.dtau, -1.0, w.ew, w.st, nb));
         CK(exp_gather(V_pool, w.offV, w.Mb, nb, (int)Mp, N, w.expV, w.st, st));
         if (mixed) CK(split_E(E, N, 0, w.cw, st));   // E slices, shared by the group
+        CKS(share_operand(h, E, N, 128, 0, w.cw.tc));
         CK(set_identity(w.U, NN, N, nb, st));
         CK(set_const(w.D, (long long)N * nb, 1.0, st));
         CK(set_identity(w.X0, NN, N, nb, st));

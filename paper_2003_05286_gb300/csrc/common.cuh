@@ -279,6 +279,42 @@ int oz_groups(int s, int N);
 // One CTA of ozaki_gemm_kernel whose loads are never issued: its bounded
 // waits run out and it ORs DQMC_STATUS_TIMEOUT into *status (device int).
 cudaError_t ozaki_selftest_timeout(int* status, cudaStream_t st);
+
+// ---------------------------------------------------------------------------
+// FP64 products as exact BF16 digit products on the tensor cores (gemm_tc.cu).
+// Digits of an operand: eight planes per 128 x 32 (left, R = 128) or 64 x 32
+// (right, R = 64) tile; a row block of the left operand is PJ = pad(N, 128)
+// rows of PM = pad(N, 32) values, of the right one pad(N, 64) columns.
+// ---------------------------------------------------------------------------
+constexpr int TC_MAX_N = 768;
+inline long long tc_plane_elems(int N, int R) {
+  return 8LL * ((N + R - 1) / R * R) * ((N + 31) / 32 * 32);
+}
+struct TcSplitArgs {
+  const double* X = nullptr; long long ldm = 1, ldj = 1, sX = 0;   // ldm or ldj is 1
+  const double* sc = nullptr; long long ssc = 0, ssc_inner = 0; int divS = 1;
+  const int* gm = nullptr; long long sgm = 0;
+  int N = 0, PJ = 0, PM = 0, R = 64;
+  __nv_bfloat16* S = nullptr; long long sS = 0;
+  int* e = nullptr; long long se = 0;
+  int b0 = 0;                                    // instance of slot 0
+  const int* lim = nullptr; int lim_at = 0;      // ended instances are left out
+};
+cudaError_t tc_split(const TcSplitArgs& a, int batch, cudaStream_t st);
+// C_b = alpha diag(rs_b) A_b B_b for the operand slots 0 .. batch - 1 holding
+// instances b0 + slot; instances with lim[b] < lim_at copy csrc_b instead.
+struct TcGemmArgs {
+  const __nv_bfloat16* A = nullptr; const int* eA = nullptr; long long sA = 0, seA = 0;
+  const __nv_bfloat16* B = nullptr; const int* eB = nullptr; long long sB = 0, seB = 0;
+  int N = 0, nkb = 0, upperA = 0, b0 = 0;
+  double* C = nullptr; long long ldc = 0, sC = 0;
+  int scaled = 0; double alpha = 1.0;            // scaled: alpha and rs apply
+  const double* rs = nullptr; long long srs = 0; int divS = 1;
+  int* status = nullptr; int status_div = 1;
+  const int* lim = nullptr; int lim_at = 0;
+  const double* csrc = nullptr; long long scsrc = 0, ldcsrc = 0;
+};
+cudaError_t tc_gemm(const TcGemmArgs& a, int batch, cudaStream_t st);
 }  // namespace dqmc
 
 // ---------------------------------------------------------------------------
