@@ -217,6 +217,7 @@ unsigned long long check_word_jacobi(bool clear);
 unsigned long long check_word_chain_small(bool clear);
 unsigned long long check_word_ozaki(bool clear);
 unsigned long long check_word_gemm_tc(bool clear);
+unsigned long long check_word_qrp_tc(bool clear);
 }  // namespace dqmc
 namespace {
 struct CheckUnit {
@@ -228,6 +229,7 @@ const CheckUnit kCheckUnits[] = {
     {"qrp_f64.cu", dqmc::check_word_qrp},     {"lu_f64.cu", dqmc::check_word_lu},
     {"jacobi_f64.cu", dqmc::check_word_jacobi}, {"chain_small.cu", dqmc::check_word_chain_small},
     {"ozaki_tc.cu", dqmc::check_word_ozaki}, {"gemm_tc.cu", dqmc::check_word_gemm_tc},
+    {"qrp_tc.cu", dqmc::check_word_qrp_tc},
 };
 #endif
 
@@ -482,6 +484,39 @@ dqmc_status share_operand(dqmc_handle h, const double* X, int N, int R, int tran
   return DQMC_OK;
 }
 
+// Slots of the blocked pivoted QR (qrp_tc.cu); without slots the factorisation
+// runs in the one-CTA kernels.
+struct QrWs {
+  char* ws = nullptr;
+  size_t bytes = 0;
+};
+
+inline bool qrtc_wanted(dqmc_handle h, int N) {
+  return !h->no_tc && h->decomp == DQMC_DECOMP_QR && N >= QRTC_MIN_N && N <= QRTC_MAX_N;
+}
+
+void take_qr(Arena& ar, long long batch, int N, int row_graded, QrWs& w) {
+  const long long slot = (long long)qrp_tc_slot_bytes(N, row_graded);
+  long long n = TC_SCRATCH / slot;
+  batch += TC_SHARES - 1;
+  n = batch < n ? batch : (n < TC_SHARES ? TC_SHARES : n);
+  w.bytes = (size_t)(n * slot);
+  w.ws = ar.take<char>(n * slot);
+}
+
+QrWs qr_part(const QrWs& w, int q, int nj, int N) {
+  const size_t slot = qrp_tc_slot_bytes(N, 0);
+  QrWs p = w;
+  p.bytes = w.bytes / slot / nj * slot;
+  p.ws += (size_t)q * p.bytes;
+  return p;
+}
+
+cudaError_t pivoted_qr(const QrpArgs& q, const QrWs& w, cudaStream_t st) {
+  const size_t slots = w.bytes ? w.bytes / qrp_tc_slot_bytes(q.N, q.Drow != nullptr) : 0;
+  return slots > 0 ? qrp_tc(q, w.ws, (int)slots, st) : qrp_f64(q, st);
+}
+
 struct ChainWs {
   double *C0, *C1, *W, *T;
   int* perm;
@@ -495,6 +530,7 @@ struct ChainWs {
   int* ozeT = nullptr;
   // FP64 chain on the tensor cores: digits, with E (or E^T) as the shared operand
   TcWs tc;
+  QrWs qr;
 };
 
 // Digit slices of E (forward chain, transposeE = 0) or E^T (backward chain)
@@ -647,7 +683,7 @@ dqmc_status chunk_qr(dqmc_handle h, int dir, int batch, int N, int k, int c, con
     CKP(PC_QRP, 8.0 / 3.0 * N * N * (double)N * batch, jacobi_svd_f64(j, st));
     return DQMC_OK;
   }
-  CKP(PC_QRP, 8.0 / 3.0 * N * N * (double)N * batch, qrp_f64(q, st));
+  CKP(PC_QRP, 8.0 / 3.0 * N * N * (double)N * batch, pivoted_qr(q, w.qr, st));
   return DQMC_OK;
 }
 
@@ -765,6 +801,7 @@ void make_sub_jobs(ChainJob* J, int nj, int dir, int batch, int N, const double*
       J[q].w.ozeT += o * cw.oz_P128;
     }
     J[q].w.tc = tc_part(cw.tc, q, nj, N);
+    J[q].w.qr = qr_part(cw.qr, q, nj, N);
     J[q].status = status + o;
     J[q].lim = lim ? lim + o : nullptr;
     o += nb;
@@ -858,6 +895,7 @@ struct TreeWs {
   int *perm, *len;
   int P0 = 1;
   TcWs tc;
+  QrWs qr;
 };
 
 int tree_width(int nc) {
@@ -947,7 +985,7 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     q.perm = w.perm; q.sperm = N;
     q.status = status; q.status_div = P0;
     q.lim = w.len; q.lim_at = 1;
-    CKP(PC_QRP, 8.0 / 3.0 * N * N * (double)N * Q, qrp_f64(q, st));
+    CKP(PC_QRP, 8.0 / 3.0 * N * N * (double)N * Q, pivoted_qr(q, w.qr, st));
     GemmArgs g;                                       // X_c = T' P^T (identity for the padding)
     g.M = g.N = g.K = N; g.batch = Q;
     g.A = w.T; g.lda = N; g.sA = NN; g.upperA = 1;
@@ -981,7 +1019,8 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     q.T = w.T; q.sT = NN;
     q.perm = w.perm; q.sperm = N;
     q.status = status; q.status_div = np;
-    CKP(PC_QRP, 8.0 / 3.0 * N * N * (double)N * B2, qrp_f64(q, st));
+    q.Drow = w.D[cur] + N; q.sDrow = 2LL * N;         // D_2
+    CKP(PC_QRP, 8.0 / 3.0 * N * N * (double)N * B2, pivoted_qr(q, w.qr, st));
     // U = U_2 u here and X = x X_1 on the aux stream, joined before the
     // next level's product reads both
     if (cudaEventRecord(fork, st) != cudaSuccess || cudaStreamWaitEvent(sx, fork, 0) != cudaSuccess)
@@ -1505,7 +1544,8 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   const long long Mp = (long long)mp_chunks * k;
   TreeWs tw;
   PlainWs pw;
-  bool tc = tc_wanted(h, N) && h->prec == DQMC_CHAIN_FP64 && (!tree || N >= TC_TREE_MIN_N);
+  const bool tc_gemms = h->prec == DQMC_CHAIN_FP64 && (!tree || N >= TC_TREE_MIN_N);
+  bool tc = !h->no_tc;
 
   auto layout = [&](Arena& ar, ExpmWs& ew, ChainWs& cw, LohWs& lw, double*& E, double*& expV,
                     double*& U, double*& D, double*& X0, double*& X1, int*& st, HostIO& io,
@@ -1516,7 +1556,9 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
     if (tree) {
       take_tree(ar, batch, N, nc, tw);
       tw.tc = TcWs{};
-      if (tc) take_tc(ar, (long long)batch * tw.P0, N, tw.tc);
+      tw.qr = QrWs{};
+      if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, (long long)batch * tw.P0, N, tw.tc);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, (long long)batch * tw.P0, N, 1, tw.qr);
       U = D = X0 = X1 = nullptr;
     } else {
       U = ar.take<double>(NN * batch);
@@ -1525,7 +1567,9 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       X1 = ar.take<double>(NN * batch);
       take_chain(ar, batch, N, cw);
       cw.tc = TcWs{};
-      if (tc) take_tc(ar, batch, N, cw.tc);
+      cw.qr = QrWs{};
+      if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, batch, N, cw.tc);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, batch, N, 0, cw.qr);
     }
     if (h->prec != DQMC_CHAIN_FP64) take_ozaki(ar, batch, N, (int)h->prec, cw);
     take_loh(ar, batch, N, lw);
@@ -2094,7 +2138,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
   double *gq[3] = {nullptr, nullptr, nullptr}, *gtmp = nullptr;   // grid values (all_tau)
   int* stat;
   int* shiftd = nullptr;
-  bool tc = tc_wanted(h, N);
+  bool tc = !h->no_tc;
   auto layout = [&](Arena& ar) {
     take_expm(ar, N, ew);
     expV = ar.take<double>(Mp * N * batch);
@@ -2109,10 +2153,15 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
     take_chain(ar, batch, N, cw);
     take_chain(ar, batch, N, cw2);
     cw.tc = cw2.tc = TcWs{};
-    if (tc) {
+    cw.qr = cw2.qr = QrWs{};
+    if (tc && tc_wanted(h, N)) {
       // the first also serves the products over all stack slots after the chains
       take_tc(ar, Q, N, cw.tc);
       take_tc(ar, batch, N, cw2.tc);
+    }
+    if (tc && qrtc_wanted(h, N)) {
+      take_qr(ar, batch, N, 0, cw.qr);
+      take_qr(ar, batch, N, 0, cw2.qr);
     }
     if (h->prec != DQMC_CHAIN_FP64) {
       take_ozaki(ar, batch, N, (int)h->prec, cw);
@@ -2260,7 +2309,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
   ExpmWs ew, ewi; ChainWs cw, cw2; StackWs sw; MidWs mw; LohWs lw; HostIO io;
   double *expV, *expmV, *Gw, *W1, *dVd = nullptr, *ldd = nullptr;
   int *stat, *sgd = nullptr;
-  bool tc = tc_wanted(h, N);
+  bool tc = !h->no_tc;
   auto layout = [&](Arena& ar) {
     take_expm(ar, N, ew);
     take_expm(ar, N, ewi);
@@ -2269,10 +2318,15 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
     take_chain(ar, batch, N, cw);
     take_chain(ar, batch, N, cw2);
     cw.tc = cw2.tc = TcWs{};
-    if (tc) {
+    cw.qr = cw2.qr = QrWs{};
+    if (tc && tc_wanted(h, N)) {
       // the first also serves the products over all stack slots after the chains
       take_tc(ar, Q, N, cw.tc);
       take_tc(ar, batch, N, cw2.tc);
+    }
+    if (tc && qrtc_wanted(h, N)) {
+      take_qr(ar, batch, N, 0, cw.qr);
+      take_qr(ar, batch, N, 0, cw2.qr);
     }
     if (h->prec != DQMC_CHAIN_FP64) {
       take_ozaki(ar, batch, N, (int)h->prec, cw);
@@ -2454,7 +2508,9 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       w.X1 = ar.take<double>(NN * nb);
       take_chain(ar, nb, N, w.cw);
       w.cw.tc = TcWs{};
+      w.cw.qr = QrWs{};
       if (tc && !mixed && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr);
       if (mixed) take_ozaki(ar, nb, N, s_digits, w.cw);
       take_loh(ar, nb, N, w.lw);
       if (h->inv == DQMC_INV_PLAIN) take_plain(ar, nb, N, w.pw);

@@ -124,10 +124,22 @@ struct QrpArgs {
   int* status = nullptr; int status_div = 1;          // nullable
   const int* lim = nullptr; int lim_at = 0;           // skip instance b when lim[b] < lim_at
   int smem_mats = 0;                                  // set by the launcher
+  // A = diag(Drow) M with Drow graded over many orders of magnitude: each row of
+  // A keeps its own relative accuracy (always so in qrp_f64).  Nullable.
+  const double* Drow = nullptr; long long sDrow = 0;
   int share_sm = 0;   // N <= 256: the register-capped kernel that fits beside an FP64 GEMM CTA
 };
 
 cudaError_t qrp_f64(const QrpArgs& a, cudaStream_t st);
+
+// The same factorisation in 32-column panels with its large products on the
+// tensor cores (qrp_tc.cu); ws holds `slots` slots of qrp_tc_slot_bytes(N, row_graded),
+// and a larger batch runs in several passes.  From N = 64 it is the faster one for
+// one instance and for 128 (figures in qrp_tc.cu); above 384 an apply's columns no
+// longer fit shared memory beside its digits.
+constexpr int QRTC_MIN_N = 64, QRTC_MAX_N = 384;
+size_t qrp_tc_slot_bytes(int N, int row_graded);
+cudaError_t qrp_tc(const QrpArgs& a, void* ws, int slots, cudaStream_t st);
 
 // One-sided Jacobi SVD, one CTA per instance (jacobi_f64.cu):
 //   A diag(Din) = U diag(D) V^T,  V^T written to Vt (row-major); W is an N x N

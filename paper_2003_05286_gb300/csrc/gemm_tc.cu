@@ -55,17 +55,12 @@ constexpr int TC_STAGE = TC_S * TC_A_TILE + TC_BSLOTS * TC_B_TILE;            //
 constexpr int TC_COPY = TC_S * (TC_A_TILE + TC_B_TILE);
 constexpr int TC_C_LD = TC_BN + 1;
 constexpr int TC_SMEM = TC_STAGES * TC_STAGE + 1024 + 128;
-constexpr int TC_NONFINITE = 1 << 20;   // exponent of a row or column with an inf or NaN
 static_assert(TC_BM * TC_C_LD * 8 <= TC_STAGES * TC_STAGE, "result tile fits the stages");
 static_assert(TC_SMEM <= 227 * 1024, "shared memory of one CTA");
 
 // BF16 A and B (K-major), FP32 accumulator, M = 128, N = 256
 constexpr uint32_t TC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) |
                               ((uint32_t)(TC_BM >> 4) << 24);
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 
 }  // namespace
 
@@ -218,12 +213,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
     long long lo[WIN >= 2 ? 32 : 1], hi[WIN >= 3 ? 32 : 1];
     bool ok = true;
     auto group4 = [](const uint32_t (&r)[4][8], int j) {
-      // |acc| <= 2^24: the conversions are exact
-      long long v = (long long)__float2int_rn(__uint_as_float(r[3][j]));
-      v += (long long)__float2int_rn(__uint_as_float(r[2][j])) * 256;
-      v += (long long)__float2int_rn(__uint_as_float(r[1][j])) * 65536;
-      v += (long long)__float2int_rn(__uint_as_float(r[0][j])) * 16777216;
-      return v;
+      return tc_group4(__uint_as_float(r[0][j]), __uint_as_float(r[1][j]), __uint_as_float(r[2][j]),
+                       __uint_as_float(r[3][j]));
     };
     if (WIN >= 2) {
 #pragma unroll
@@ -334,11 +325,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
 // One CTA per 32 rows j of one instance.  Phase 1 stages them in shared memory
 // (lanes along the contiguous index: j when ldj = 1, else m) and finds each
 // row's largest exponent; phase 2 gives every thread eight consecutive m of one
-// j, i.e. one 16-byte store per digit.  Adding 0x80 to every byte of the
-// fixed-point value turns its bytes into the balanced digits plus 128, and a
-// byte becomes BF16 through the FP32 number 2^23 + byte: about 30 integer and
-// FP32 instructions per entry, and the kernel is bound by its stores
-// (16 bytes per entry).
+// j, i.e. one 16-byte store per digit: about 30 integer and FP32 instructions
+// per entry, and the kernel is bound by its stores (16 bytes per entry).
 // ---------------------------------------------------------------------------
 template <bool ALONG_M>
 __global__ void __launch_bounds__(256) tc_split_kernel(const TcSplitArgs a) {
@@ -410,9 +398,7 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const TcSplitArgs a) {
     int m2 = emax[0][tid];
     if (!ALONG_M)
       for (int r = 1; r < 8; ++r) m2 = max(m2, emax[r][tid]);
-    // biased exponent m2: entries are below 2^{m2 - 1022}, scaled by
-    // 2^{-(m2 - 1020)} they lie in (-1/4, 1/4); denormal entries count as zero
-    const int e = m2 == 0 ? 0 : (m2 == 0x7ff ? TC_NONFINITE : m2 - 1020);
+    const int e = tc_exponent(m2);
     emax[0][tid] = e;
     a.e[(long long)z * a.se + j0 + tid] = e;
   }
@@ -424,39 +410,13 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const TcSplitArgs a) {
     const int jj = it & 31, kb = it >> 5;
     const int e = emax[0][jj];
     const int mb = kb * 32 + ch * 8;
-    uint32_t glo[8], ghi[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const long long bits = __double_as_longlong(tile[(mb + k) * 33 + jj]);
-      const int E = (int)((bits >> 52) & 0x7ff);
-      unsigned long long F = 0;              // |x| 2^{64 - e}, below 2^62
-      if (E != 0 && e < TC_NONFINITE) {
-        const unsigned long long m53 = ((unsigned long long)bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-        const int sh = E - 1011 - e;         // at most 9
-        F = sh >= 0 ? m53 << sh : (sh > -55 ? (m53 + (1ull << (-sh - 1))) >> -sh : 0ull);
-      }
-      const unsigned long long G =
-          (bits < 0 ? 0ull - F : F) + 0x8080808080808080ull;   // bytes: digits + 128
-      glo[k] = (uint32_t)G;
-      ghi[k] = (uint32_t)(G >> 32);
-    }
     const int jr = (j0 + jj) % a.R;
     __nv_bfloat16* out = S + ((long long)((j0 + jj) / a.R) * nkb + kb) * (TC_S * (long long)plane) +
                          jr * 32 + ((ch ^ ((jr >> 1) & 3)) << 3);   // 64-byte swizzle
-#pragma unroll
-    for (int q = 0; q < TC_S; ++q) {
-      uint32_t w[4];
-#pragma unroll
-      for (int k = 0; k < 8; k += 2) {
-        const uint32_t sel = 0x7440u | (uint32_t)(q < 4 ? 3 - q : 7 - q);
-        const float f0 = __uint_as_float(__byte_perm(q < 4 ? ghi[k] : glo[k], 0x4B000000u, sel)) - 8388736.0f;
-        const float f1 =
-            __uint_as_float(__byte_perm(q < 4 ? ghi[k + 1] : glo[k + 1], 0x4B000000u, sel)) - 8388736.0f;
-        w[k >> 1] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632u);
-      }
+    tc_digits8(e, [&](int k) { return tile[(mb + k) * 33 + jj]; }, [&](int q, uint4 w) {
       if (DQMC_CHECK((reinterpret_cast<uintptr_t>(out + q * plane) & 15) == 0, q))
-        *reinterpret_cast<uint4*>(out + q * plane) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
+        *reinterpret_cast<uint4*>(out + q * plane) = w;
+    });
   }
 }
 

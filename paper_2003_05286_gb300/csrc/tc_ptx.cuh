@@ -139,4 +139,75 @@ __device__ __forceinline__ double split_times_pow2(long long T, unsigned int r, 
                                           (mant & 0xFFFFFFFFFFFFFull)));
 }
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Exponent e that brings entries whose largest biased exponent is E into
+// (-1/4, 1/4) as x 2^{-e}; a column without a normal entry keeps 0, one with an
+// inf or NaN gets TC_NONFINITE.
+constexpr int TC_NONFINITE = 1 << 20;
+__device__ __forceinline__ int tc_exponent(int E) {
+  return E == 0 ? 0 : (E == 0x7ff ? TC_NONFINITE : E - 1020);
+}
+
+// The eight balanced base-256 digits of V (4 or 8) consecutive values (FP64
+// bits, value k scaled by 2^{-ex(k)} into (-1/4, 1/4) and rounded to a multiple of 2^-64),
+// as V BF16 per digit: store(q, words) with the digits q of the V values.
+// Adding 0x80 to every byte of the fixed-point value turns its bytes into the
+// digits plus 128, and a byte becomes BF16 through the FP32 number 2^23 + byte.
+template <int V, class Load, class Exp, class Store>
+__device__ __forceinline__ void tc_digits(Exp&& ex, Load&& load, Store&& store) {
+  uint32_t glo[V], ghi[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const long long bits = __double_as_longlong(load(k));
+    const int E = (int)((bits >> 52) & 0x7ff);
+    unsigned long long F = 0;              // |x| 2^{64 - e}, below 2^62
+    const int e = ex(k);
+    if (E != 0 && E != 0x7ff && e < TC_NONFINITE / 2) {
+      const unsigned long long m53 = ((unsigned long long)bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+      const int sh = E - 1011 - e;         // at most 9
+      F = sh >= 0 ? m53 << (sh < 10 ? sh : 10) : (sh > -55 ? (m53 + (1ull << (-sh - 1))) >> -sh : 0ull);
+    }
+    const unsigned long long G = (bits < 0 ? 0ull - F : F) + 0x8080808080808080ull;
+    glo[k] = (uint32_t)G;
+    ghi[k] = (uint32_t)(G >> 32);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    uint32_t w[V / 2];
+    const uint32_t sel = 0x7440u | (uint32_t)(q < 4 ? 3 - q : 7 - q);
+#pragma unroll
+    for (int k = 0; k < V; k += 2) {
+      const float f0 =
+          __uint_as_float(__byte_perm(q < 4 ? ghi[k] : glo[k], 0x4B000000u, sel)) - 8388736.0f;
+      const float f1 =
+          __uint_as_float(__byte_perm(q < 4 ? ghi[k + 1] : glo[k + 1], 0x4B000000u, sel)) - 8388736.0f;
+      w[k >> 1] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632u);
+    }
+    store(q, w);
+  }
+}
+
+template <class Load, class Store>
+__device__ __forceinline__ void tc_digits8(int e, Load&& load, Store&& store) {
+  tc_digits<8>([e](int) { return e; }, load, [&](int q, const uint32_t (&w)[4]) { store(q, make_uint4(w[0], w[1], w[2], w[3])); });
+}
+
+template <class Load, class Store>
+__device__ __forceinline__ void tc_digits4(int e, Load&& load, Store&& store) {
+  tc_digits<4>([e](int) { return e; }, load, [&](int q, const uint32_t (&w)[2]) { store(q, make_uint2(w[0], w[1])); });
+}
+
+// Four accumulators of adjacent weights as one integer in units of the last
+// (|acc| <= 2^24: the conversions are exact).
+__device__ __forceinline__ long long tc_group4(float a0, float a1, float a2, float a3) {
+  long long v = (long long)__float2int_rn(a3);
+  v += (long long)__float2int_rn(a2) * 256;
+  v += (long long)__float2int_rn(a1) * 65536;
+  v += (long long)__float2int_rn(a0) * 16777216;
+  return v;
+}
+
 }  // namespace dqmc
