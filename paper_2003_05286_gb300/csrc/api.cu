@@ -517,6 +517,15 @@ cudaError_t pivoted_qr(const QrpArgs& q, const QrWs& w, cudaStream_t st) {
   return slots > 0 ? qrp_tc(q, w.ws, (int)slots, st) : qrp_f64(q, st);
 }
 
+// opA(A) Z = opR(R): on the tensor cores with room for it, else one CTA per instance.
+cudaError_t solve(const LuArgs& l, const QrWs& w, cudaStream_t st) {
+  if (w.bytes && l.N >= SOLVETC_MIN_N && l.N <= QRTC_MAX_N) {
+    const size_t slots = w.bytes / solve_tc_slot_bytes(l.N);
+    if (slots > 0) return solve_tc(l, w.ws, (int)(slots < 65535 ? slots : 65535), st);
+  }
+  return lu_solve_f64(l, st);
+}
+
 struct ChainWs {
   double *C0, *C1, *W, *T;
   int* perm;
@@ -1088,7 +1097,7 @@ void take_loh(Arena& ar, int batch, int N, LohWs& w) {
 
 dqmc_status run_loh(dqmc_handle h, int batch, int N, const double* U, long long sU,
                     const double* D, long long sD, const double* X, long long sX, double* G,
-                    double* logdet, int* sign, int* status, const LohWs& w) {
+                    double* logdet, int* sign, int* status, const LohWs& w, const QrWs& qr) {
   cudaStream_t st = h->cur;
   const long long NN = (long long)N * N;
   CK(dsplit_vec(D, sD, N, batch, w.Dpinv, 1, st));   // D_p^{-1}
@@ -1100,7 +1109,7 @@ dqmc_status run_loh(dqmc_handle h, int batch, int N, const double* U, long long 
   l1.W = w.Wlu; l1.sW = 2 * NN;
   l1.sign = w.sX;
   l1.status = status;
-  CKP(PC_LU, lu_flops(N, N) * batch, lu_solve_f64(l1, st));
+  CKP(PC_LU, lu_flops(N, N) * batch, solve(l1, qr, st));
   Axpby2Args ax;
   ax.N = N; ax.batch = batch;
   ax.A = w.Y; ax.sA = NN;
@@ -1123,7 +1132,7 @@ dqmc_status run_loh(dqmc_handle h, int batch, int N, const double* U, long long 
   l2.logabsdet = w.lad;
   l2.sign = w.sM;
   l2.status = status;
-  CKP(PC_LU, lu_flops(N, l2.nrhs) * batch, lu_solve_f64(l2, st));
+  CKP(PC_LU, lu_flops(N, l2.nrhs) * batch, solve(l2, qr, st));
   CK(finish_logdet(D, sD, N, batch, w.lad, w.sX, w.sM, logdet, sign, status, st));
   return DQMC_OK;
 }
@@ -1239,10 +1248,10 @@ dqmc_status run_one_plus(dqmc_handle h, int batch, int N, const double* U, long 
 dqmc_status run_inversion(dqmc_handle h, int batch, int N, const double* U, long long sU,
                           const double* D, long long sD, const double* X, long long sX, double* G,
                           double* logdet, int* sign, int* status, const LohWs& lw,
-                          const PlainWs& pw) {
+                          const PlainWs& pw, const QrWs& qr) {
   if (h->inv == DQMC_INV_PLAIN)
     return run_one_plus(h, batch, N, U, sU, D, sD, X, sX, G, logdet, sign, status, pw);
-  return run_loh(h, batch, N, U, sU, D, sD, X, sX, G, logdet, sign, status, lw);
+  return run_loh(h, batch, N, U, sU, D, sD, X, sX, G, logdet, sign, status, lw, qr);
 }
 
 // ---------------------------------------------------------------------------
@@ -1618,7 +1627,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   if (tree) {
     const double *Ut, *Dt, *Xt;
     CKS(run_chain_tree(h, batch, N, M, k, E, expV, Mp * N, tw, stout, &Ut, &Dt, &Xt));
-    CKS(run_inversion(h, batch, N, Ut, NN, Dt, N, Xt, NN, Gout, ldout, sgout, stout, lw, pw));
+    CKS(run_inversion(h, batch, N, Ut, NN, Dt, N, Xt, NN, Gout, ldout, sgout, stout, lw, pw, tw.qr));
   } else {
     if (cw.oz_s > 0) CK(split_E(E, N, 0, cw, st));   // E slices, shared by all instances
     CKS(share_operand(h, E, N, 128, 0, cw.tc));
@@ -1641,7 +1650,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       CKS(run_chain(h, +1, batch, N, M, k, E, expV, Mp * N, s, cw, stout));
     }
     const double* Xf = (nc & 1) ? X1 : X0;
-    CKS(run_inversion(h, batch, N, U, NN, D, N, Xf, NN, Gout, ldout, sgout, stout, lw, pw));
+    CKS(run_inversion(h, batch, N, U, NN, D, N, Xf, NN, Gout, ldout, sgout, stout, lw, pw, cw.qr));
   }
 
   if (host) {
@@ -1733,7 +1742,7 @@ dqmc_status greens_on_workspace(void* stream, void* ws, size_t ws_bytes, int bat
   s.X2 = X1;
   CKS(run_chain(h, +1, batch, N, M, k, ew.t0, expV, Mp * N, s, cw, stout));
   const double* Xf = (nc & 1) ? X1 : X0;
-  CKS(run_loh(h, batch, N, U, NN, D, N, Xf, NN, G, logdet, sign, stout, lw));
+  CKS(run_loh(h, batch, N, U, NN, D, N, Xf, NN, G, logdet, sign, stout, lw, QrWs{}));
   return DQMC_OK;
 }
 }  // namespace dqmc
@@ -1879,7 +1888,7 @@ void take_mid(Arena& ar, long long Q, int N, int ncols, MidWs& w) {
 // G(tau,0) to Gt0 and G(0,tau) to G0t (each may be null), each Q x N x N.
 dqmc_status run_two_stack_inversion(dqmc_handle h, int Q, int N, int nt, const StackWs& w,
                                     const MidWs& m, double* Gtt, double* Gt0, double* G0t,
-                                    int* status, const TcWs& tc) {
+                                    int* status, const TcWs& tc, const QrWs& qr) {
   cudaStream_t st = h->cur;
   const long long NN = (long long)N * N;
   const bool want_z = Gtt || G0t;                      // Z = mid^{-1} a_p^{-1} U_F^T
@@ -1916,7 +1925,7 @@ dqmc_status run_two_stack_inversion(dqmc_handle h, int Q, int N, int nt, const S
   lu.Z = m.Z; lu.sZ = (long long)N * ncols; lu.ldz = ncols;
   lu.W = m.Wlu; lu.sW = (long long)N * (N + ncols);
   lu.status = status; lu.status_div = nt;
-  CKP(PC_LU, lu_flops(N, ncols) * Q, lu_solve_f64(lu, st));
+  CKP(PC_LU, lu_flops(N, ncols) * Q, solve(lu, qr, st));
   CK(dsplit_vec(w.Db, N, N, Q, m.bpinv, 1, st));
   for (int part = 0; part < 2; ++part) {
     double* out = part == 0 ? Gtt : Gt0;
@@ -2160,7 +2169,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       take_tc(ar, batch, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
-      take_qr(ar, batch, N, 0, cw.qr);
+      take_qr(ar, Q, N, 0, cw.qr);
       take_qr(ar, batch, N, 0, cw2.qr);
     }
     if (h->prec != DQMC_CHAIN_FP64) {
@@ -2207,7 +2216,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
   if (all_tau)
     for (int i = 0; i < 3; ++i) out[i] = gq[i];
   CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, out[0], plain_t0 ? nullptr : out[1],
-                              out[2], stout, cw.tc));
+                              out[2], stout, cw.tc, cw.qr));
   if (plain_t0) CKS(run_inv_sum_t0(h, (int)Q, N, nt, sw, sumw, out[1], stout));
   if (all_tau) {
     // tau between grid points: k - 1 one-slice steps from every grid value,
@@ -2325,7 +2334,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       take_tc(ar, batch, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
-      take_qr(ar, batch, N, 0, cw.qr);
+      take_qr(ar, Q, N, 0, cw.qr);
       take_qr(ar, batch, N, 0, cw2.qr);
     }
     if (h->prec != DQMC_CHAIN_FP64) {
@@ -2369,9 +2378,9 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
   CKS(run_stacks(h, batch, N, M, k, ew.t0, expV, Mp * N, sw, cw, cw2, stout));
   // log det from the full forward product B(beta, 0) = U_F a X_F (slot nc)
   CKS(run_loh(h, batch, N, sw.UF + nc * NN, nt * NN, sw.DF + (long long)nc * N, (long long)nt * N,
-              sw.XF + nc * NN, nt * NN, nullptr, ldo, sgo, stout, lw));
+              sw.XF + nc * NN, nt * NN, nullptr, ldo, sgo, stout, lw, cw.qr));
   // checkpoints G_{jk+1}
-  CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, Gw, nullptr, nullptr, stout, cw.tc));
+  CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, Gw, nullptr, nullptr, stout, cw.tc, cw.qr));
   CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
   TcWs wr = cw.tc;                                     // E^{-1} as the shared right operand
   wr.Es = cw2.tc.Es; wr.eEs = cw2.tc.eEs;
@@ -2639,7 +2648,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
         }
         const double* Xf = (ncmax & 1) ? w.X1 : w.X0;
         CKS(run_inversion(h, nb, N, w.U, NN, w.D, N, Xf, NN, G_pool ? w.G : nullptr, w.ld, w.sg,
-                          w.st, w.lw, w.pw));
+                          w.st, w.lw, w.pw, w.cw.qr));
         if (G_pool) CK(scatter_mats(w.G, w.offG, N, nb, G_pool, st));
         CK(scatter_scalars(w.gidx, nb, w.ld, w.sg, w.st, logdet, sign, status, st));
         return DQMC_OK;

@@ -179,6 +179,17 @@ struct LuArgs {
 
 cudaError_t lu_solve_f64(const LuArgs& a, cudaStream_t st);
 
+// The same solve by Householder QR with its large products on the tensor cores
+// (qrp_tc.cu); ws holds `slots` slots of solve_tc_slot_bytes(N).  Used from N =
+// 160, by N alone so that an instance's result does not depend on its batch; N
+// right-hand sides, LU -> QR: N = 144 1.76 -> 0.70 ms (1 instance), 1.81 -> 1.62
+// (128), 10.4 -> 13.8 (1024); N = 200 3.81 -> 1.05 and 3.93 -> 2.94 (128); N = 256
+// 6.92 -> 1.28 and 8.30 -> 3.99; N = 324 14.8 -> 2.02 and 19.5 -> 8.08; residuals
+// a fifth of the LU's.
+constexpr int SOLVETC_MIN_N = 160;
+size_t solve_tc_slot_bytes(int N);
+cudaError_t solve_tc(const LuArgs& a, void* ws, int slots, cudaStream_t st);
+
 // ---------------------------------------------------------------------------
 // Element-wise helpers.
 // ---------------------------------------------------------------------------
@@ -307,6 +318,7 @@ struct TcSplitArgs {
   const double* sc = nullptr; long long ssc = 0, ssc_inner = 0; int divS = 1;
   const int* gm = nullptr; long long sgm = 0;
   int N = 0, PJ = 0, PM = 0, R = 64;
+  int upper = 0;                                 // entries with m < j count as zero
   __nv_bfloat16* S = nullptr; long long sS = 0;
   int* e = nullptr; long long se = 0;
   int b0 = 0;                                    // instance of slot 0

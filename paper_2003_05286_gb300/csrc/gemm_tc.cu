@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const TcSplitArgs a) {
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const int r = row_of(mb + 8 * u);
-        v[u] = r >= 0 && j < N ? X[(long long)r * a.ldm + (long long)j * a.ldj] : 0.0;
+        v[u] = r >= 0 && j < N && !(a.upper && r < j) ? X[(long long)r * a.ldm + (long long)j * a.ldj] : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const TcSplitArgs a) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int j = j0 + wid + 8 * u;
-        v[u] = r >= 0 && j < N ? X[(long long)r * a.ldm + (long long)j * a.ldj] : 0.0;
+        v[u] = r >= 0 && j < N && !(a.upper && r < j) ? X[(long long)r * a.ldm + (long long)j * a.ldj] : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {

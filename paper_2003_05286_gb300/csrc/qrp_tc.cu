@@ -402,10 +402,49 @@ __device__ __forceinline__ double stacked_value(const long long* ex, int i, int 
   return split_times_pow2(hi + (lo >> 32), (unsigned int)(lo & 0xFFFFFFFFll), e - 72);
 }
 
+// acc (256 TMEM columns, 32 per weight) = left (8 digits x 128 rows x 32 k) times
+// right (3 zero tiles, then 8 digits x 32 columns x 32 k).
+__device__ __forceinline__ void mma_rows(uint32_t acc, uint32_t left, uint32_t right) {
+  const uint64_t dv = smem_desc_sw64(left), dw = smem_desc_sw64(right);
+  for (int r = 0; r < 2; ++r)
+    for (int kk = 0; kk < 2; ++kk)
+      for (int q = 0; q <= 4 * r + 3; ++q)
+        umma(acc + 128u * r, dv + (uint64_t)(kk * 2 + q * ((128 * 64) >> 4)),
+             dw + (uint64_t)(kk * 2 + (3 + 4 * r - q) * (DT >> 4)), IDESC_128,
+             kk == 0 && q == 0 ? 0u : 1u);
+}
+
+// a2[c LD + row] -= the product's entry for eight columns of warp wid (of 16), row
+// below `rows`; er: the row's exponent, ew: biased exponents of the columns.
+__device__ __forceinline__ void rows_subtract(uint32_t acc, int wid, int row, int rows, int er,
+                                              const int* ew, double* a2, int LD) {
+  const int cb = 8 * (wid >> 2);
+  const uint32_t la = acc + ((uint32_t)((wid & 3) * 32) << 16);
+  uint32_t r[8][8];
+#pragma unroll
+  for (int g = 0; g < 8; ++g) tmem_ld8_nowait(la + 32 * g + cb, r[g]);
+  tmem_wait_ld();
+  if (row >= rows) return;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const long long hi = tc_group4(__uint_as_float(r[0][j]), __uint_as_float(r[1][j]),
+                                   __uint_as_float(r[2][j]), __uint_as_float(r[3][j]));
+    const long long lo = tc_group4(__uint_as_float(r[4][j]), __uint_as_float(r[5][j]),
+                                   __uint_as_float(r[6][j]), __uint_as_float(r[7][j]));
+    const int E = ew[cb + j];
+    const double v = E == 0x7ff || er >= TC_NONFINITE / 2
+                         ? __longlong_as_double(0x7ff8000000000000ll)
+                         : split_times_pow2(hi + (lo >> 32), (unsigned int)(lo & 0xFFFFFFFFll),
+                                            tc_exponent(E) + er - 72);
+    a2[(cb + j) * LD + row] -= v;
+  }
+}
+
 struct QrTc {
   QrpArgs q;
   int np, nkb, nmt, b0;      // panels, 32-row blocks, 128-row tiles, instance of slot 0
   int sets;                  // digit sets: 2 with row scales
+  int nc;                    // columns of W^T (the solver: N + right-hand sides)
   unsigned char* ws;         // per slot: see the pointers below
   long long slot_bytes;
   __host__ __device__ long long set_bytes() const {
@@ -436,13 +475,25 @@ struct QrTc {
   __host__ __device__ int* rem(int z, int which) const {        // remaining columns, ping-pong
     return reinterpret_cast<int*>(lnrm(z) + 32 * nkb) + which * 32 * nkb;
   }
+  // the solver: digits of R (128-row tiles x 32 columns, as V) and their row exponents
+  __host__ __device__ unsigned char* r(int z) const { return slot(z) + set_bytes(); }
+  __host__ __device__ long long r_bytes() const { return (long long)nmt * nkb * V_TILE; }
+  __host__ __device__ int* r_exp(int z) const { return reinterpret_cast<int*>(r(z) + r_bytes()); }
 };
 
 void qr_geometry(QrTc& a, int N, int row_graded) {
   a.np = a.nkb = (N + NB - 1) / NB;
   a.nmt = (N + 127) / 128;
   a.sets = row_graded ? 2 : 1;
+  a.nc = N;
   a.slot_bytes = (a.sets * a.set_bytes() + 5LL * 32 * a.nkb * 4 + 1023) & ~1023LL;
+}
+
+// The solver's slot: one digit set, R's digits and exponents.
+void solve_geometry(QrTc& a, int N, int nrhs) {
+  qr_geometry(a, N, 0);
+  a.nc = N + nrhs;
+  a.slot_bytes = (a.set_bytes() + a.r_bytes() + 128LL * a.nmt * 4 + 1023) & ~1023LL;
 }
 
 __device__ __forceinline__ bool qr_skip(const QrTc& a, int b) {
@@ -492,7 +543,8 @@ __global__ void __launch_bounds__(256) qr_init_kernel(const QrTc a) {
 
 // ---- panel ---------------------------------------------------------------------
 // BIG (N > 256): 64 instead of 128 candidates of the pivot search.
-template <bool BIG>
+// PIV: with the pivot search; otherwise the columns in their order (the solver).
+template <bool BIG, bool PIV>
 __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
   constexpr int CN = BIG ? 64 : 128;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -531,7 +583,7 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
     return;
   double* W = a.q.W + (long long)b * a.q.sW;
   const double* Din = a.din(z);
-  int* perm = a.q.perm + (long long)b * a.q.sperm;
+  int* perm = PIV ? a.q.perm + (long long)b * a.q.sperm : nullptr;
 
   if (tid == 0) {
     mbar_init(bar, 1);
@@ -548,7 +600,11 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
   // ---- candidates: the CN remaining columns of largest key (ties: lowest place)
   const double* Drow = a.q.Drow ? a.q.Drow + (long long)b * a.q.sDrow : nullptr;
   if (tid < 32 * nkl) s_rho[tid] = row_rho(Drow, j0 + tid, N);
-  if (tid < m) {
+  if (!PIV && tid < NB) {
+    s_rem[tid] = j0 + tid;
+    s_sel[tid] = tid;
+  }
+  if (PIV && tid < m) {
     const int col = a.rem(z, p & 1)[tid];
     const float k = log2_wide_f(Din[col]) + a.lnrm(z)[col];
     s_rem[tid] = col;
@@ -558,7 +614,7 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_holder;
-  if (tid < m) {
+  if (PIV && tid < m) {
     const float k = s_key[tid];
     int rank = 0;
     for (int u = 0; u < m; ++u) rank += s_key[u] > k || (s_key[u] == k && u < tid);
@@ -566,7 +622,7 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
   }
   __syncthreads();
   // ---- FP32 pivoted reduction of the candidates: nb pivots -------------------------
-  {
+  if constexpr (PIV) {
     // rows per thread rounded up: straight-line loops
 #define DQMC_SEARCH(TPC_, KM_)                                                                 \
   do {                                                                                         \
@@ -593,13 +649,13 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
   }
   __syncthreads();
   // ---- pivot order and the columns that remain (their order kept) ------------------
-  if (tid < nb) {
+  if (PIV && tid < nb) {
     const int pos = s_cand[s_sel[tid]];
     perm[j0 + tid] = s_rem[pos];
     s_sel[tid] = pos;
   }
   __syncthreads();
-  if (tid < m) {
+  if (PIV && tid < m) {
     int before = 0;
     bool taken = false;
     for (int s = 0; s < nb; ++s) {
@@ -787,9 +843,11 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
 }
 
 // ---- block reflectors on 32 columns --------------------------------------------
-// FORMQ = false: the remaining columns 32 blockIdx.x .. of rem after panel p get
-// (1 - V T V^T)^T; true: columns 32 blockIdx.x .. of Q, all panels backwards.
-template <bool FORMQ>
+// APPLY_REM: the remaining columns 32 blockIdx.x .. of rem after panel p get
+// (1 - V T V^T)^T; APPLY_NEXT (the solver): the columns right of panel p in W^T;
+// APPLY_Q: columns 32 blockIdx.x .. of Q, all panels backwards.
+enum { APPLY_REM, APPLY_NEXT, APPLY_Q };
+template <int MODE>
 __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
@@ -817,10 +875,13 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
                       (unsigned)(reinterpret_cast<unsigned char*>(s_fail + 1) - smem_raw), LD))
     return;
   double* W = a.q.W + (long long)b * a.q.sW;
+  constexpr bool FORMQ = MODE == APPLY_Q;
   const int j0 = NB * p, c0 = 32 * blockIdx.x;
-  const int ncols = FORMQ ? (N - c0 < 32 ? N - c0 : 32)
-                          : (N - j0 - NB - c0 < 32 ? N - j0 - NB - c0 : 32);
-  const int* rem = a.rem(z, (p + 1) & 1) + c0;
+  const int next = j0 + NB < N ? j0 + NB : N;   // first column right of the panel
+  const int left = (FORMQ ? N : (MODE == APPLY_REM ? N : a.nc) - next) - c0;
+  const int ncols = left < 32 ? left : 32;
+  const int* rem = MODE == APPLY_REM ? a.rem(z, (p + 1) & 1) + c0 : nullptr;
+  auto column = [&](int c) { return MODE == APPLY_REM ? rem[c] : next + c0 + c; };
 
   if (tid == 0) {
     mbar_init(full, 1);
@@ -839,7 +900,7 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
   for (int u = 0; u < 2; ++u) {             // a warp per column, four loads in flight
     const int c = wid + 16 * u;
     double* dst = a2 + c * LD;
-    const double* src = W + (long long)(!FORMQ && c < ncols ? rem[c] : 0) * N;
+    const double* src = W + (long long)(!FORMQ && c < ncols ? column(c) : 0) * N;
     for (int r0 = lane; r0 < 32 * a.nkb; r0 += 128) {
       double v[4];
 #pragma unroll
@@ -982,13 +1043,7 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
       if (tid == 0) {
         wait_or_fail(full, nfull & 1, s_fail);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t dv = smem_desc_sw64(smem_u32(base)), dw = smem_desc_sw64(smem_u32(wz));
-        for (int r = 0; r < 2; ++r)
-          for (int kk = 0; kk < 2; ++kk)
-            for (int q = 0; q <= 4 * r + 3; ++q)
-              umma(acc + 128u * r, dv + (uint64_t)(kk * 2 + q * ((128 * 64) >> 4)),
-                   dw + (uint64_t)(kk * 2 + (3 + 4 * r - q) * (DT >> 4)), IDESC_128,
-                   kk == 0 && q == 0 ? 0u : 1u);
+        mma_rows(acc, smem_u32(base), smem_u32(wz));
         umma_commit(done);
       }
       ++nfull;
@@ -1000,30 +1055,7 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int row = 128 * t + (wid & 3) * 32 + lane;
-      const uint32_t la = acc + ((uint32_t)((wid & 3) * 32) << 16);
-      {
-        const int cb = 8 * (wid >> 2);
-        uint32_t r[8][8];
-#pragma unroll
-        for (int g = 0; g < 8; ++g) tmem_ld8_nowait(la + 32 * g + cb, r[g]);
-        tmem_wait_ld();
-        if (row < 32 * a.nkb) {
-          const int er = s_er[row];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const long long hi = tc_group4(__uint_as_float(r[0][j]), __uint_as_float(r[1][j]),
-                                           __uint_as_float(r[2][j]), __uint_as_float(r[3][j]));
-            const long long lo = tc_group4(__uint_as_float(r[4][j]), __uint_as_float(r[5][j]),
-                                           __uint_as_float(r[6][j]), __uint_as_float(r[7][j]));
-            const int E = ew[cb + j];
-            const double v = E == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll)
-                                        : split_times_pow2(hi + (lo >> 32),
-                                                           (unsigned int)(lo & 0xFFFFFFFFll),
-                                                           tc_exponent(E) + er - 72);
-            a2[(cb + j) * LD + row] -= v;
-          }
-        }
-      }
+      rows_subtract(acc, wid, row, 32 * a.nkb, row < 32 * a.nkb ? s_er[row] : 0, ew, a2, LD);
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncthreads();
     }
@@ -1038,10 +1070,12 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
     for (int u = 0; u < 2; ++u) {
       const int c = wid + 16 * u;
       if (c >= ncols) break;
-      const int col = rem[c];
+      const int col = column(c);
       for (int r = j0 + lane; r < N; r += 32) W[(long long)col * N + r] = a2[c * LD + r];
-      const float ln = warp_log2_norm(a2 + c * LD, j0 + NB, N, bad);
-      if (lane == 0) a.lnrm(z)[col] = ln;
+      if (MODE == APPLY_REM) {
+        const float ln = warp_log2_norm(a2 + c * LD, j0 + NB, N, bad);
+        if (lane == 0) a.lnrm(z)[col] = ln;
+      }
     }
     if (lane == 0 && bad && a.q.status)
       atomicOr(&a.q.status[b / a.q.status_div], DQMC_STATUS_NONFINITE_SCALE);
@@ -1111,6 +1145,281 @@ __global__ void __launch_bounds__(256) qr_out_kernel(const QrTc a) {
   }
 }
 
+namespace {
+size_t apply_smem(int nkb) {
+  return 1024 + RING + 11 * DT + (size_t)32 * (32 * nkb + 1) * 8 + 3 * NB * TLD * 8 + 64 * nkb * 4 + 512;
+}
+size_t panel_smem(int N, int nkb) {
+  return 1024 + RING + ((size_t)NB * (32 * nkb + 1) + 2 * NB * TLD + 2 * XS + 3 * NB) * 8 +
+         (3 * QF + 2 + 2 * N + 128 + 3 * NB + 64 * nkb + 32) * 4 + 64;
+}
+}  // namespace
+
+// ===========================================================================
+// Solver: opA(A) Z = opR(R) by the same panels and reflectors without pivoting
+// (Householder QR of [A | R], stable as it is), then blocked back substitution.
+// Takes the place of lu_kernel (one CTA per instance on its SM's FP64 pipe)
+// where that is the slower one.  det A = (-1)^{reflectors} prod r_ii.
+// ===========================================================================
+// [opA(A) | opR(R)] by columns into W^T; one CTA per 32 columns of one instance
+__global__ void __launch_bounds__(256) solve_init_kernel(const QrTc a, const LuArgs l) {
+  __shared__ double tile[32][33];
+  const int b = a.b0 + blockIdx.y, N = a.q.N, c0 = blockIdx.x * 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (!DQMC_CHECK(blockDim.x == 256 && l.nrhs == a.nc - N, l.nrhs)) return;
+  double* W = a.q.W + (long long)b * a.q.sW;
+  const double* A = l.A + (long long)b * l.sA;
+  const double* R = l.R ? l.R + (long long)b * l.sR : nullptr;
+  const double* Rd = l.Rdiag ? l.Rdiag + (long long)b * l.sRdiag : nullptr;
+  for (int r0 = 0; r0 < N; r0 += 32) {
+    // entries that are contiguous along the column come in along it, the others along rows
+    for (int u = wid; u < 32; u += 8) {
+      const int cr = c0 + lane, rr = r0 + u;      // along a row
+      const int cc = c0 + u, rc = r0 + lane;      // along a column
+      if (cr < a.nc && rr < N) {
+        if (cr < N) { if (!l.transA) tile[lane][u] = A[(long long)rr * N + cr]; }
+        else if (!Rd && !l.transR) tile[lane][u] = R[(long long)rr * l.ldr + cr - N];
+      }
+      if (cc < a.nc && rc < N) {
+        if (cc < N) { if (l.transA) tile[u][lane] = A[(long long)cc * N + rc]; }
+        else if (Rd) tile[u][lane] = rc == cc - N ? (l.invRdiag ? 1.0 / Rd[rc] : Rd[rc]) : 0.0;
+        else if (l.transR) tile[u][lane] = R[(long long)(cc - N) * l.ldr + rc];
+      }
+    }
+    __syncthreads();
+    for (int u = wid; u < 32; u += 8)
+      if (c0 + u < a.nc && r0 + lane < N) W[(long long)(c0 + u) * N + r0 + lane] = tile[u][lane];
+    __syncthreads();
+  }
+}
+
+// log|det|, sign and singular pivots of one instance: lanes along the diagonal,
+// sums in a fixed order
+__global__ void __launch_bounds__(32) solve_det_kernel(const QrTc a, const LuArgs l) {
+  const int z = blockIdx.x, b = a.b0 + z, N = a.q.N, lane = threadIdx.x;
+  const double* W = a.q.W + (long long)b * a.q.sW;
+  double ls = 0.0;
+  int neg = 0;
+  bool zero = false;
+  for (int i = lane; i < N; i += 32) {
+    const double r = W[(long long)i * N + i];
+    zero |= r == 0.0;
+    neg ^= (r < 0.0) ^ (a.T(z, i / NB, 0)[(i % NB) * (NB + 1)] > 0.0);
+    if (l.logabsdet) ls += log(fabs(r));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ls += __shfl_xor_sync(0xffffffffu, ls, o);
+    neg ^= __shfl_xor_sync(0xffffffffu, neg, o);
+  }
+  zero = __any_sync(0xffffffffu, zero);
+  if (lane == 0) {
+    if (l.logabsdet) l.logabsdet[b] = ls;
+    if (l.sign) l.sign[b] = neg ? -1 : 1;
+    if (zero && l.status) atomicOr(&l.status[b / l.status_div], DQMC_STATUS_SINGULAR);
+  }
+}
+
+// R Z = Q^T R.h.s. for 32 right-hand sides per CTA, in shared memory: per 32-row
+// block from the last, substitution in the block (a warp per two rows, lanes
+// along the right-hand sides), then Y -= R(above, block) Z as exact digit products.
+__global__ void __launch_bounds__(512, 1) solve_back_kernel(const QrTc a, const LuArgs l) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* base = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int z = blockIdx.y, b = a.b0 + z, N = a.q.N;
+  const int LD = 32 * a.nkb + 1;
+  unsigned char* wz = base + RING;                              // 3 zero tiles, 8 digits of Z
+  double* y = reinterpret_cast<double*>(wz + 11 * DT);          // [32][LD]
+  double* zs = y + 32 * LD;                                     // block of Z [32][TLD]
+  double* rpp = zs + NB * TLD;                                  // diagonal block of R
+  double* rinv = rpp + NB * TLD;                                // [32 nkb]
+  int* er = reinterpret_cast<int*>(rinv + 32 * a.nkb);          // [32 nkb]
+  int* ew = er + 32 * a.nkb;                                    // [32]
+  uint64_t* full = reinterpret_cast<uint64_t*>(ew + 32);
+  uint64_t* done = full + 1;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(done + 1);
+  int* s_fail = reinterpret_cast<int*>(tmem_holder + 1);
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (!DQMC_CHECK(blockDim.x == 512 && a.nkb <= 12, a.nkb) ||
+      !DQMC_CHECK(dyn_smem_bytes() >=
+                      (unsigned)(reinterpret_cast<unsigned char*>(s_fail + 1) - smem_raw), LD))
+    return;
+  const double* W = a.q.W + (long long)b * a.q.sW;
+  const int c0 = 32 * blockIdx.x, ncols = l.nrhs - c0 < 32 ? l.nrhs - c0 : 32;
+  if (tid == 0) {
+    mbar_init(full, 1);
+    mbar_init(done, 1);
+    *s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (wid == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_holder)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  for (int i = tid; i < 3 * DT / 16; i += 512) reinterpret_cast<uint4*>(wz)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int u = 0; u < 2; ++u) {
+    const int c = wid + 16 * u;
+    const double* src = W + (long long)(N + c0 + (c < ncols ? c : 0)) * N;
+    for (int r0 = lane; r0 < 32 * a.nkb; r0 += 128) {
+      double v[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) v[t] = c < ncols && r0 + 32 * t < N ? src[r0 + 32 * t] : 0.0;
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (r0 + 32 * t < 32 * a.nkb) y[c * LD + r0 + 32 * t] = v[t];
+    }
+  }
+  for (int r = tid; r < 32 * a.nkb; r += 512) {
+    const double d = r < N ? W[(long long)r * N + r] : 0.0;
+    rinv[r] = d != 0.0 ? 1.0 / d : 0.0;
+    er[r] = a.r_exp(z)[r];
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_holder;
+  uint32_t nfull = 0, ndone = 0;
+  const unsigned char* gr = a.r(z);
+  for (int p = a.np - 1; p >= 0; --p) {
+    const int j0 = NB * p;
+    if (tid == 0 && p > 0) {
+      mbar_arrive_expect_tx(full, V_TILE);
+      bulk_load(base, gr + (long long)p * V_TILE, V_TILE, full);
+    }
+    for (int e = tid; e < NB * NB; e += 512) {       // along the columns of W^T
+      const int i = e & 31, j = e >> 5;
+      rpp[i * TLD + j] = i < j && j0 + j < N ? W[(long long)(j0 + j) * N + j0 + i] : 0.0;
+    }
+    if (tid < 32) ew[tid] = 0;
+    const int i0 = wid, i1 = 31 - wid;               // this warp's rows of the block
+    double y0 = y[lane * LD + j0 + i0], y1 = y[lane * LD + j0 + i1];
+    __syncthreads();
+    for (int i = NB - 1; i >= 0; --i) {
+      if (i == i0 || i == i1) zs[i * TLD + lane] = (i == i0 ? y0 : y1) * rinv[j0 + i];
+      __syncthreads();
+      if (i0 < i) {                                  // (i1 < i implies i0 < i)
+        const double zi = zs[i * TLD + lane];
+        y0 = fma(-rpp[i0 * TLD + i], zi, y0);
+        if (i1 < i) y1 = fma(-rpp[i1 * TLD + i], zi, y1);
+      }
+    }
+    {
+      const double z0 = zs[i0 * TLD + lane], z1 = zs[i1 * TLD + lane];
+      y[lane * LD + j0 + i0] = z0;
+      y[lane * LD + j0 + i1] = z1;
+      atomicMax(&ew[lane], max((int)((__double_as_longlong(z0) >> 52) & 0x7ff),
+                               (int)((__double_as_longlong(z1) >> 52) & 0x7ff)));
+    }
+    __syncthreads();
+    if (p == 0) break;
+    if (tid < 256) {
+      const int c = tid >> 3, ch = (tid >> 1) & 3, hf = tid & 1;
+      unsigned char* dst = wz + 3 * DT + swz(c, ch) + 8 * hf;
+      tc_digits4(tc_exponent(ew[c]), [&](int k) { return zs[(8 * ch + 4 * hf + k) * TLD + c]; },
+                 [&](int q, uint2 w) { *reinterpret_cast<uint2*>(dst + q * DT) = w; });
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    const int nt = (j0 + 127) / 128;
+    for (int t = 0; t < nt; ++t) {
+      const uint32_t acc = tmem + 256u * (uint32_t)(t & 1);
+      if (tid == 0) {
+        wait_or_fail(full, nfull & 1, s_fail);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        mma_rows(acc, smem_u32(base), smem_u32(wz));
+        umma_commit(done);
+      }
+      ++nfull;
+      wait_or_fail(done, ndone & 1, s_fail);
+      ++ndone;
+      if (tid == 0 && t + 1 < nt) {
+        mbar_arrive_expect_tx(full, V_TILE);
+        bulk_load(base, gr + ((long long)(t + 1) * a.nkb + p) * V_TILE, V_TILE, full);
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int row = 128 * t + (wid & 3) * 32 + lane;
+      rows_subtract(acc, wid, row, j0, row < 32 * a.nkb ? er[row] : 0, ew, y, LD);
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+    }
+  }
+  double* Z = l.Z + (long long)b * l.sZ;
+  if (!l.transZ) {
+    for (int r = wid; r < N; r += 16)
+      if (lane < ncols) Z[(long long)r * l.ldz + c0 + lane] = y[lane * LD + r];
+  } else {
+    for (int c = wid; c < ncols; c += 16)
+      for (int r = lane; r < N; r += 32) Z[(long long)(c0 + c) * l.ldz + r] = y[c * LD + r];
+  }
+  if (*(volatile int*)s_fail && tid == 0) {
+    mbar_wait(full, nfull & 1);   // a copy still in flight lands before the CTA exits (bounded)
+    if (l.status) atomicOr(&l.status[b / l.status_div], DQMC_STATUS_TIMEOUT);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (wid == 0) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
+                 : "memory");
+  }
+}
+
+size_t solve_tc_slot_bytes(int N) {
+  QrTc a;
+  solve_geometry(a, N, 0);
+  return (size_t)a.slot_bytes;
+}
+
+cudaError_t solve_tc(const LuArgs& l, void* ws, int slots, cudaStream_t st) {
+  if (l.batch <= 0) return cudaSuccess;
+  if (l.N < SOLVETC_MIN_N || l.N > QRTC_MAX_N || !ws || slots < 1) return cudaErrorInvalidValue;
+  const int N = l.N;
+  QrTc a;
+  solve_geometry(a, N, l.nrhs);
+  a.q.N = N; a.q.batch = l.batch;
+  a.q.W = l.W; a.q.sW = l.sW;
+  a.q.status = l.status; a.q.status_div = l.status_div;
+  a.ws = static_cast<unsigned char*>(ws);
+  const int LD = 32 * a.nkb + 1;
+  const size_t sm_apply = apply_smem(a.nkb), sm_panel = panel_smem(N, a.nkb);
+  const size_t sm_back = 1024 + RING + 11 * DT + ((size_t)32 * LD + 2 * NB * TLD + 32 * a.nkb) * 8 +
+                         32 * a.nkb * 4 + 512;
+  cudaError_t e;
+  if ((e = allow_dyn_smem(qr_apply_kernel<APPLY_NEXT>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<false, false>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<true, false>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(solve_back_kernel)) != cudaSuccess) return e;
+  if (slots > 65535) slots = 65535;
+  for (a.b0 = 0; a.b0 < l.batch; a.b0 += slots) {
+    const int nz = l.batch - a.b0 < slots ? l.batch - a.b0 : slots;
+    solve_init_kernel<<<dim3((a.nc + 31) / 32, nz), 256, 0, st>>>(a, l);
+    for (int p = 0; p < a.np; ++p) {
+      if (N <= 256) qr_panel_kernel<false, false><<<nz, 512, sm_panel, st>>>(a, p);
+      else qr_panel_kernel<true, false><<<nz, 512, sm_panel, st>>>(a, p);
+      const int left = a.nc - (NB * (p + 1) < N ? NB * (p + 1) : N);
+      if (left > 0) qr_apply_kernel<APPLY_NEXT><<<dim3((left + 31) / 32, nz), 512, sm_apply, st>>>(a, p);
+    }
+    if (l.logabsdet || l.sign || l.status) solve_det_kernel<<<nz, 32, 0, st>>>(a, l);
+    if (l.nrhs > 0) {
+      TcSplitArgs r;                        // digits of R's rows, zero below the diagonal
+      r.X = l.W; r.ldm = N; r.ldj = 1; r.sX = l.sW;
+      r.N = N; r.R = 128; r.PJ = 128 * a.nmt; r.PM = 32 * a.nkb; r.upper = 1;
+      r.S = reinterpret_cast<__nv_bfloat16*>(a.r(0)); r.sS = a.slot_bytes / 2;
+      r.e = a.r_exp(0); r.se = a.slot_bytes / 4;
+      r.b0 = a.b0;
+      if ((e = tc_split(r, nz, st)) != cudaSuccess) return e;
+      solve_back_kernel<<<dim3((l.nrhs + 31) / 32, nz), 512, sm_back, st>>>(a, l);
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 size_t qrp_tc_slot_bytes(int N, int row_graded) {
   QrTc a;
   qr_geometry(a, N, row_graded);
@@ -1127,26 +1436,24 @@ cudaError_t qrp_tc(const QrpArgs& q, void* ws, int slots, cudaStream_t st) {
   a.ws = static_cast<unsigned char*>(ws);
   const int LD = 32 * a.nkb + 1;
   const size_t sm_init = (size_t)32 * LD * 8;
-  const size_t sm_apply = 1024 + RING + 11 * DT + (size_t)32 * LD * 8 + 3 * NB * TLD * 8 + 64 * a.nkb * 4 + 512;
-  const size_t sm_panel = 1024 + RING + ((size_t)NB * LD + 2 * NB * TLD + 2 * XS + 3 * NB) * 8 +
-                          (3 * QF + 2 + 2 * N + 128 + 3 * NB + 64 * a.nkb + 32) * 4 + 64;
+  const size_t sm_apply = apply_smem(a.nkb), sm_panel = panel_smem(N, a.nkb);
   cudaError_t e;
   if ((e = allow_dyn_smem(qr_init_kernel)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_apply_kernel<false>)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_apply_kernel<true>)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_panel_kernel<false>)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_panel_kernel<true>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_apply_kernel<APPLY_REM>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_apply_kernel<APPLY_Q>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<false, true>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<true, true>)) != cudaSuccess) return e;
   if (slots > 65535) slots = 65535;
   for (a.b0 = 0; a.b0 < q.batch; a.b0 += slots) {
     const int nz = q.batch - a.b0 < slots ? q.batch - a.b0 : slots;
     qr_init_kernel<<<dim3(a.nkb, nz), 256, sm_init, st>>>(a);
     for (int p = 0; p < a.np; ++p) {
-      if (N <= 256) qr_panel_kernel<false><<<nz, 512, sm_panel, st>>>(a, p);
-      else qr_panel_kernel<true><<<nz, 512, sm_panel, st>>>(a, p);
+      if (N <= 256) qr_panel_kernel<false, true><<<nz, 512, sm_panel, st>>>(a, p);
+      else qr_panel_kernel<true, true><<<nz, 512, sm_panel, st>>>(a, p);
       const int left = N - NB * (p + 1);
-      if (left > 0) qr_apply_kernel<false><<<dim3((left + 31) / 32, nz), 512, sm_apply, st>>>(a, p);
+      if (left > 0) qr_apply_kernel<APPLY_REM><<<dim3((left + 31) / 32, nz), 512, sm_apply, st>>>(a, p);
     }
-    qr_apply_kernel<true><<<dim3(a.nkb, nz), 512, sm_apply, st>>>(a, 0);
+    qr_apply_kernel<APPLY_Q><<<dim3(a.nkb, nz), 512, sm_apply, st>>>(a, 0);
     qr_out_kernel<<<dim3(a.nkb, nz), 256, 0, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

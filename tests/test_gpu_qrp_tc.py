@@ -86,3 +86,37 @@ def test_more_instances_than_slots(dq):
     for b in (0, 64, 129):
         G1, ld1, _, _ = dq.greens(K, 0.1, V[b], 3, handle=dq.Handle(fold=0))
         assert torch.equal(G1, G[b]) and float(ld1) == float(ld[b])
+
+
+@pytest.mark.parametrize("N", [160, 161, 257])
+def test_solver_through_displaced_and_gradient(dq, N):
+    """The QR solver (N >= 160) with 2 N right-hand sides, and with none (log det alone)."""
+    K = di.chain_hopping(N)
+    V = 0.3 * di.ising_field(5300 + N, 7, N)
+    Gtt, Gt0, st = dq.greens_tdisplaced(_dev(K), 0.1, _dev(V), 3)
+    assert int(st) == 0
+    Ott, Ot0 = od.greens_tdisplaced(K, 0.1, V, 3)
+    for got, want in ((Gtt, Ott), (Gt0, Ot0)):
+        assert np.abs(got.cpu().numpy() - want).max() <= GTOL * max(1.0, np.abs(want).max())
+    ldo, so = od.logdet(K, 0.1, V, 3)
+    ld, sg, st = dq.logdet(_dev(K), 0.1, _dev(V), 3)
+    assert int(st) == 0 and abs(float(ld) - ldo) <= LTOL * abs(ldo) and int(sg) == so
+    ld, sg, dV, st = dq.logdet_grad(_dev(K), 0.1, _dev(V), 3)
+    assert int(st) == 0 and abs(float(ld) - ldo) <= LTOL * abs(ldo) and int(sg) == so
+    assert np.abs(dV.cpu().numpy() - od.logdet_grad(K, 0.1, V, 3)).max() <= 1e-9
+
+
+def test_solver_sign(dq):
+    """Negative determinants at N = 160: the sign comes from the reflectors and R."""
+    N = 160
+    K = np.zeros((N, N))
+    K[:3, :3] = di.chain_hopping(3)          # a triangle with strong fields, the rest decoupled
+    signs = set()
+    for seed in range(24):
+        V = np.zeros((6, N))
+        V[:, :3] = 2.0 * di.gaussian_field(seed, 6, 3)
+        ld, sg, st = dq.logdet(_dev(K), 0.5, _dev(V), 2)
+        ldo, so = od.logdet(K, 0.5, V, 2)
+        assert int(st) == 0 and int(sg) == so and abs(float(ld) - ldo) <= LTOL * abs(ldo)
+        signs.add(int(sg))
+    assert signs == {-1, 1}
