@@ -25,10 +25,12 @@
 // lose relative digits, as they do in the QR that consumes the products.
 // A row or column with a non-finite entry gives NaN throughout.
 //
-// Measured against DFMA tiles at 92% of the FP64 pipe's rate: the equal-time
-// step of 128 instances at N = 256, M = 200 takes 252 ms instead of 925 (its
-// products about 70 instead of 700), the gradient of 64 instances at N = 144
-// 126 ms instead of 346, both with the same error against 64-bit references.
+// Measured against DFMA tiles at 92% of the FP64 pipe's rate: one product of 128
+// instances at N = 256 takes 170 us (and its operand's split 43) instead of 3430,
+// with the same error of the whole chain against 64-bit references.  A CTA of
+// that product spends 29 thousand cycles in the MMAs (95% of their rate at N =
+// 256 columns, a quarter of it on zero tiles), 10 in the conversion of the sums
+// (21 with eight epilogue warps and branches in the rounding) and 5 around them.
 //
 // Digits are stored as tiles (128 rows x 32 k for the left operand, 64 x 32
 // for the right), the eight planes of a tile adjacent, each in the 64-byte
@@ -46,7 +48,7 @@ namespace {
 constexpr int TC_S = 8;            // digits per operand
 constexpr int TC_BM = 128, TC_BN = 64, TC_BK = 32;
 constexpr int TC_STAGES = 2;
-constexpr int TC_EPI = 256;        // epilogue threads (8 warps); + producer and MMA warps
+constexpr int TC_EPI = 512;        // epilogue threads (16 warps); + producer and MMA warps
 constexpr int TC_THREADS = TC_EPI + 64;
 constexpr int TC_A_TILE = TC_BM * TC_BK * 2, TC_B_TILE = TC_BN * TC_BK * 2;   // bytes of one digit
 constexpr int TC_BZERO = 3;        // zero tiles in front of the right operand's digits
@@ -64,8 +66,8 @@ constexpr uint32_t TC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) 
 
 }  // namespace
 
-// One CTA: a 128 x 64 tile of one product.  Warps 0-7 epilogue (two per TMEM
-// lane quarter), warp 8 copies, warp 9 allocates TMEM and issues the MMAs.
+// One CTA: a 128 x 64 tile of one product.  Warps 0-15 epilogue (four per
+// TMEM lane quarter), warp 16 copies, warp 17 allocates TMEM and issues the MMAs.
 // An accumulator block r holds groups 4r .. 4r + 3 in 256 TMEM columns; each
 // MMA has N = 256 and adds, for one left digit p, the right digits 4r - p ..
 // 4r - p + 3 (zero tiles where there is none), so consecutive MMAs write the
@@ -121,7 +123,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
     *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 9) {
+  if (warp == 17) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_holder)),
                  "r"(512u)
@@ -139,7 +141,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_holder;
 
-  if (warp == 8) {
+  if (warp == 16) {
     if (lane == 0) {
       const __nv_bfloat16* a0 = a.A + (long long)z * a.sA +
                                 ((long long)blockIdx.y * a.nkb + kb0) * (TC_S * TC_BM * TC_BK);
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
           mbar_wait(&full[i % TC_STAGES], (i / TC_STAGES) & 1);
     }
     __syncwarp();
-  } else if (warp == 9) {
+  } else if (warp == 17) {
     if (lane == 0) {
       bool ok = true;
       for (int i = 0; i < nk && ok; ++i) {
@@ -207,10 +209,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
   } else {
     // ---- epilogue ------------------------------------------------------------
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
-    const int cbase = (warp >> 2) * 32;
+    const int cbase = (warp >> 2) * 16;
     const int rl = (warp & 3) * 32 + lane, row = m0 + rl;
     const int nwin = (nk + 3) / 4;             // windows of block 1 (block 0: every second)
-    long long lo[WIN >= 2 ? 32 : 1], hi[WIN >= 3 ? 32 : 1];
+    long long lo[WIN >= 2 ? 16 : 1], hi[WIN >= 3 ? 16 : 1];
     bool ok = true;
     auto group4 = [](const uint32_t (&r)[4][8], int j) {
       return tc_group4(__uint_as_float(r[0][j]), __uint_as_float(r[1][j]), __uint_as_float(r[2][j]),
@@ -218,7 +220,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
     };
     if (WIN >= 2) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
+      for (int j = 0; j < 16; ++j) {
         lo[WIN >= 2 ? j : 0] = 0;
         if (WIN >= 3) hi[WIN >= 3 ? j : 0] = 0;
       }
@@ -230,7 +232,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < 2; ++c) {
           uint32_t r[4][8];
 #pragma unroll
           for (int g = 0; g < 4; ++g)
@@ -244,7 +246,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
         if (lane == 0) mbar_arrive(&acc_free[1]);
         if (WIN >= 3 && both) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
+          for (int c = 0; c < 2; ++c) {
             uint32_t r[4][8];
 #pragma unroll
             for (int g = 0; g < 4; ++g)
@@ -273,18 +275,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
       if (a.rs && row < N) rscale *= a.rs[(long long)(b / a.divS) * a.srs + row];
       double* ctile = reinterpret_cast<double*>(base);   // the stages are idle now
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        uint32_t rh[4][8], rl4[4][8];
+      for (int c = 0; c < 2; ++c) {
+        uint32_t r[4][8];
+        long long l8[8];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          tmem_ld8_nowait(tmem + lane_addr + g * TC_BN + cbase + 8 * c, rh[g]);
-          tmem_ld8_nowait(tmem + lane_addr + (4 + g) * TC_BN + cbase + 8 * c, rl4[g]);
-        }
+        for (int g = 0; g < 4; ++g) tmem_ld8_nowait(tmem + lane_addr + (4 + g) * TC_BN + cbase + 8 * c, r[g]);
         tmem_wait_ld();
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          long long h = group4(rh, j), l = group4(rl4, j);
-          if (WIN >= 2) l += lo[WIN >= 2 ? 8 * c + j : 0];
+          l8[j] = group4(r, j);
+          if (WIN >= 2) l8[j] += lo[WIN >= 2 ? 8 * c + j : 0];
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) tmem_ld8_nowait(tmem + lane_addr + g * TC_BN + cbase + 8 * c, r[g]);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          long long h = group4(r, j);
+          const long long l = l8[j];
           if (WIN >= 3) h += hi[WIN >= 3 ? 8 * c + j : 0];
           const int col = n0 + cbase + 8 * c + j;
           const int eb = col < N ? eB[col] : 0;
@@ -297,7 +305,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
       }
       if (a.scaled) {   // row scale (and alpha): one FP64 multiply per entry
 #pragma unroll 4
-        for (int j = 0; j < 32; ++j) ctile[rl * TC_C_LD + cbase + j] *= rscale;
+        for (int j = 0; j < 16; ++j) ctile[rl * TC_C_LD + cbase + j] *= rscale;
       }
       asm volatile("bar.sync 1, %0;" ::"r"(TC_EPI) : "memory");
       double* Cb = a.C + (long long)b * a.sC;
@@ -311,7 +319,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
-  if (warp == 9) {
+  if (warp == 17) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
                  : "memory");

@@ -3,7 +3,9 @@
 // instructions, and the integer-only rounding of an exact digit sum to FP64.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 namespace dqmc {
 
@@ -101,42 +103,47 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// (T 2^32 + r) 2^e correctly rounded to FP64, for |T| < 2^45 and 0 <= r < 2^32
-// (the exact sum of the weight groups), with 64-bit integer operations only:
-// the magnitude is split into (Ta, ra) the same way, the 53-bit mantissa taken
-// from Ta and the top bits of ra, and the discarded bits of ra decide the
-// round-to-nearest-even step.
-__device__ __forceinline__ double split_times_pow2(long long T, unsigned int r, int e) {
-  if (T == 0 && r == 0) return 0.0;
-  const bool neg = T < 0;
-  unsigned long long Ta;
-  unsigned int ra;
-  if (!neg) { Ta = (unsigned long long)T; ra = r; }
-  else if (r) { Ta = (unsigned long long)(-(T + 1)); ra = (unsigned int)(0x100000000ull - r); }
-  else { Ta = (unsigned long long)(-T); ra = 0u; }
-  unsigned long long mant;
-  int ex;
-  if (Ta < (1ull << 21)) {   // below 2^53: exact
-    const unsigned long long A = (Ta << 32) | ra;
-    const int nb = 64 - __clzll((long long)A);
-    mant = A << (53 - nb);
-    ex = nb - 1 + e;
-  } else {                   // 54..77 bits: drop sh = 1..24 bits of ra
-    const int nb = 96 - __clzll((long long)Ta);
-    const int sh = nb - 53;
-    mant = (Ta << (32 - sh)) | (ra >> sh);
-    const unsigned int rem = ra & ((1u << sh) - 1u), half = 1u << (sh - 1);
-    ex = nb - 1 + e;
-    if (rem > half || (rem == half && (mant & 1ull))) {
-      if (++mant == (1ull << 53)) { mant >>= 1; ++ex; }
-    }
-  }
-  const int be = ex + 1023;
-  if (be <= 0 || be >= 2047)   // result outside the normal range: scale in FP64
-    return ldexp((double)Ta * 4294967296.0 + (double)ra, e) * (neg ? -1.0 : 1.0);
-  return __longlong_as_double((long long)((neg ? (1ull << 63) : 0ull) |
-                                          ((unsigned long long)be << 52) |
-                                          (mant & 0xFFFFFFFFFFFFFull)));
+// (T 2^32 + r) 2^e correctly rounded to FP64, for |T| < 2^62 and 0 <= r < 2^32
+// (the exact sum of the weight groups), with 32-bit integer operations and no
+// branch but for results outside the normal range: the FP64 pipe stays free, and
+// a CTA's epilogue converts thousands of sums.  The magnitude's three words are
+// moved up past leading zero words and shifted to a leading one; the 53 top bits
+// and the biased exponent less one are added, so that the leading one completes
+// the exponent, and the round-to-nearest-even increment may carry into it.
+__host__ __device__ __forceinline__ double split_times_pow2(long long T, unsigned int r, int e) {
+  const unsigned int neg = (unsigned int)((unsigned long long)T >> 63);
+  const unsigned int w0n = neg ? 0u - r : r;
+  const unsigned long long Tm = neg ? ~(unsigned long long)T + (r == 0u) : (unsigned long long)T;
+  unsigned int w2 = (unsigned int)(Tm >> 32), w1 = (unsigned int)Tm, w0 = w0n;
+  int be = e + 95 + 1022;                    // biased exponent of the leading bit, less one
+  if (w2 == 0u) { w2 = w1; w1 = w0; w0 = 0u; be -= 32; }
+  if (w2 == 0u) { w2 = w1; w1 = 0u; be -= 32; }
+#ifdef __CUDA_ARCH__
+  const int lz = __clz((int)w2);
+  const unsigned int m1 = __funnelshift_l(w1, w2, lz), m0 = __funnelshift_l(w0, w1, lz);
+#else
+  const int lz = w2 ? __builtin_clz(w2) : 32;
+  const unsigned long long h = ((unsigned long long)w2 << 32) | w1, q = ((unsigned long long)w1 << 32) | w0;
+  const unsigned int m1 = lz < 32 ? (unsigned int)((h << lz) >> 32) : w1;
+  const unsigned int m0 = lz < 32 ? (unsigned int)((q << lz) >> 32) : w0;
+#endif
+  const unsigned int low = w0 << (lz & 31);  // (w0 is zero wherever lz reaches 32)
+  be -= lz;
+  const unsigned int up = (m0 & 0x400u) && ((m0 & 0xBFFu) | low) ? 1u : 0u;
+  unsigned long long bits = ((unsigned long long)((unsigned int)be << 20) << 32) +
+                            (((unsigned long long)(m1 >> 11)) << 32) +
+                            (unsigned long long)((m1 << 21) | (m0 >> 11)) + up;
+  bits |= (unsigned long long)neg << 63;
+  if (w2 == 0u) bits = 0ull;
+  else if (be < 1 || be > 2044)              // result outside the normal range: scale in FP64
+    return ldexp((double)Tm * 4294967296.0 + (double)w0n, e) * (neg ? -1.0 : 1.0);
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)bits);
+#else
+  double d;
+  memcpy(&d, &bits, 8);
+  return d;
+#endif
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
