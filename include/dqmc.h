@@ -78,6 +78,8 @@ enum dqmc_status_bits {
  * scales), the digit products accumulate exactly in FP32 on the tcgen05
  * tensor cores and are recombined in FP64; a product is accurate to about
  * N 2^{-7s-1} of (row max x column max), normwise rather than elementwise.
+ * From N = 64 the FP64 products themselves run on the tensor cores (eight
+ * base-256 digits, about N 2^{-58}), and DQMC_CHAIN_BF16X8 uses them.
  * Supported for N <= 256 in dqmc_greens, dqmc_logdet, dqmc_greens_tdisplaced,
  * dqmc_logdet_grad (both stacks) and dqmc_greens_ragged (every instance N <= 256);
  * N > 256 returns DQMC_ERR_UNSUPPORTED (dqmc_greens_noalloc takes no handle

@@ -393,6 +393,16 @@ inline bool tc_wanted(dqmc_handle h, int N) {
   return !h->no_tc && N >= TC_MIN_N && N <= TC_MAX_N;
 }
 
+// Digits of the reduced-precision chain (ozaki_tc.cu), 0 for products in FP64
+// accuracy.  Eight BF16 digits per operand are what the FP64 products take too,
+// with 8 instead of 7 bits each: DQMC_CHAIN_BF16X8 runs on them wherever they
+// serve (one product of 128 instances, N = 256: 218 -> 170 us, its split 79 ->
+// 43, error 2^-58 instead of 2^-51 of row max x column max).
+inline int reduced_digits(dqmc_handle h, int N) {
+  if (h->prec == DQMC_CHAIN_FP64) return 0;
+  return h->prec == DQMC_CHAIN_BF16X8 && tc_wanted(h, N) ? 0 : (int)h->prec;
+}
+
 void take_tc(Arena& ar, long long batch, int N, TcWs& w) {
   const long long ea = tc_plane_elems(N, 128), eb = tc_plane_elems(N, 64);
   long long cap = TC_SCRATCH / (2 * (ea + eb));
@@ -824,12 +834,13 @@ bool pipeline_enabled() {
 }
 
 // Number of staggered sub-batches of an equal-time chain: DQMC_PIPELINE=n
-// (2..8) overrides the default (2 for FP64 products, 4 for tensor-core ones).
+// (2..8) overrides the default of 2 (N = 256, 128 instances, 2 / 3 / 4 / 8: 128 /
+// 129 / 130 / 149 ms; reduced precision 142 / 141 / 143 / 165).
 constexpr int kMaxJobs = TC_SHARES;
-int pipeline_jobs(bool mixed) {
+int pipeline_jobs() {
   const char* e = getenv("DQMC_PIPELINE");
   if (e && e[0] >= '2' && e[0] <= '8' && e[1] == 0) return e[0] - '0';
-  return mixed ? 4 : 2;
+  return 2;
 }
 
 // The jobs run on aux streams sbase .. sbase + nj - 1, forked from and joined
@@ -1453,7 +1464,7 @@ static dqmc_status graph_call(dqmc_handle h, GraphKey key, F&& body) {
   key.add((unsigned long long)h->fold);
   key.add((unsigned long long)h->inv);
   key.add((unsigned long long)h->decomp);
-  key.add((unsigned long long)pipeline_enabled() * 16 + (unsigned long long)pipeline_jobs(h->prec != DQMC_CHAIN_FP64));
+  key.add((unsigned long long)pipeline_enabled() * 16 + (unsigned long long)pipeline_jobs());
   key.addp(h->ws);
   key.addp(h->stream);
   bool same = h->gvalid && h->gexec && key.n <= 24;
@@ -1553,7 +1564,8 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   const long long Mp = (long long)mp_chunks * k;
   TreeWs tw;
   PlainWs pw;
-  const bool tc_gemms = h->prec == DQMC_CHAIN_FP64 && (!tree || N >= TC_TREE_MIN_N);
+  const int digits = reduced_digits(h, N);
+  const bool tc_gemms = digits == 0 && (!tree || N >= TC_TREE_MIN_N);
   bool tc = !h->no_tc;
 
   auto layout = [&](Arena& ar, ExpmWs& ew, ChainWs& cw, LohWs& lw, double*& E, double*& expV,
@@ -1580,7 +1592,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, batch, N, cw.tc);
       if (tc && qrtc_wanted(h, N)) take_qr(ar, batch, N, 0, cw.qr);
     }
-    if (h->prec != DQMC_CHAIN_FP64) take_ozaki(ar, batch, N, (int)h->prec, cw);
+    if (digits) take_ozaki(ar, batch, N, digits, cw);
     take_loh(ar, batch, N, lw);
     if (h->inv == DQMC_INV_PLAIN) take_plain(ar, batch, N, pw);
     st = ar.take<int>(batch);
@@ -1639,7 +1651,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
     s.D = D; s.slotD = 0; s.instD = N;
     s.X = X0; s.slotX = 0; s.instX = NN;
     s.X2 = X1;
-    const int nj = pipeline_jobs(cw.oz_s > 0);
+    const int nj = pipeline_jobs();
     if (batch >= 4 * nj && pipeline_enabled()) {
       // nj sub-batches on nj streams, product phases staggered so that the QRs
       // of some sub-batches run while the others multiply
@@ -2172,9 +2184,9 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       take_qr(ar, Q, N, 0, cw.qr);
       take_qr(ar, batch, N, 0, cw2.qr);
     }
-    if (h->prec != DQMC_CHAIN_FP64) {
-      take_ozaki(ar, batch, N, (int)h->prec, cw);
-      take_ozaki(ar, batch, N, (int)h->prec, cw2);
+    if (const int digits = reduced_digits(h, N)) {
+      take_ozaki(ar, batch, N, digits, cw);
+      take_ozaki(ar, batch, N, digits, cw2);
     }
     take_stacks(ar, batch, N, nt, sw);
     take_mid(ar, Q, N, ncols > 0 ? ncols : N, mw);
@@ -2337,9 +2349,9 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       take_qr(ar, Q, N, 0, cw.qr);
       take_qr(ar, batch, N, 0, cw2.qr);
     }
-    if (h->prec != DQMC_CHAIN_FP64) {
-      take_ozaki(ar, batch, N, (int)h->prec, cw);
-      take_ozaki(ar, batch, N, (int)h->prec, cw2);
+    if (const int digits = reduced_digits(h, N)) {
+      take_ozaki(ar, batch, N, digits, cw);
+      take_ozaki(ar, batch, N, digits, cw2);
     }
     take_stacks(ar, batch, N, nt, sw);
     take_mid(ar, Q, N, N, mw);
@@ -2498,7 +2510,6 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
     g->idx.push_back(b);
     if (d.M > g->Mmax) g->Mmax = d.M;
   }
-  const int s_digits = mixed ? (int)h->prec : 0;
   // ---- workspace (h->ws) and index tables (h->rtab): one region per group ----
   std::vector<RaggedGroupWs> gw(groups.size());
   bool tc = true;
@@ -2518,9 +2529,10 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       take_chain(ar, nb, N, w.cw);
       w.cw.tc = TcWs{};
       w.cw.qr = QrWs{};
-      if (tc && !mixed && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
+      const int digits = reduced_digits(h, N);
+      if (tc && !digits && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
       if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr);
-      if (mixed) take_ozaki(ar, nb, N, s_digits, w.cw);
+      if (digits) take_ozaki(ar, nb, N, digits, w.cw);
       take_loh(ar, nb, N, w.lw);
       if (h->inv == DQMC_INV_PLAIN) take_plain(ar, nb, N, w.pw);
       w.G = ar.take<double>(NN * nb);
@@ -2588,7 +2600,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
   // ---- streams and the fork event (created outside any capture) --------------
   // up to 8 group slots; a slot has its group's stream and nj more for the
   // staggered sub-batches of a group large enough to pipeline
-  const int nj = pipeline_jobs(mixed);
+  const int nj = pipeline_jobs();
   const size_t nslots = groups.size() < 8 ? groups.size() : 8;
   const size_t per_slot = (size_t)nj + 1;
   const size_t nstreams = nslots * per_slot;
@@ -2627,7 +2639,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
         const double* E = E_pool ? E_pool + g.offK : w.ew.t0;
         if (!E_pool) CKS(run_expm(h, K_pool + g.offK, N, g.dtau, -1.0, w.ew, w.st, nb));
         CK(exp_gather(V_pool, w.offV, w.Mb, nb, (int)Mp, N, w.expV, w.st, st));
-        if (mixed) CK(split_E(E, N, 0, w.cw, st));   // E slices, shared by the group
+        if (w.cw.oz_s > 0) CK(split_E(E, N, 0, w.cw, st));   // E slices, shared by the group
         CKS(share_operand(h, E, N, 128, 0, w.cw.tc));
         CK(set_identity(w.U, NN, N, nb, st));
         CK(set_const(w.D, (long long)N * nb, 1.0, st));

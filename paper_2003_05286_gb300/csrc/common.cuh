@@ -134,10 +134,11 @@ cudaError_t qrp_f64(const QrpArgs& a, cudaStream_t st);
 
 // The same factorisation in 32-column panels with its large products on the
 // tensor cores (qrp_tc.cu); ws holds `slots` slots of qrp_tc_slot_bytes(N, row_graded),
-// and a larger batch runs in several passes.  From N = 64 it is the faster one for
-// one instance and for 128 (figures in qrp_tc.cu); above 384 an apply's columns no
+// and a larger batch runs in several passes.  From N = 48 it is the faster one for
+// one instance and for 128 (N = 40 0.239 -> 0.212 and 0.239 -> 0.248 ms, N = 48
+// 0.308 -> 0.229 and 0.310 -> 0.264; more in qrp_tc.cu); above 384 an apply's columns no
 // longer fit shared memory beside its digits.
-constexpr int QRTC_MIN_N = 64, QRTC_MAX_N = 384;
+constexpr int QRTC_MIN_N = 48, QRTC_MAX_N = 384;
 size_t qrp_tc_slot_bytes(int N, int row_graded);
 cudaError_t qrp_tc(const QrpArgs& a, void* ws, int slots, cudaStream_t st);
 
