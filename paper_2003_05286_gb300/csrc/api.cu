@@ -218,6 +218,7 @@ unsigned long long check_word_chain_small(bool clear);
 unsigned long long check_word_ozaki(bool clear);
 unsigned long long check_word_gemm_tc(bool clear);
 unsigned long long check_word_qrp_tc(bool clear);
+unsigned long long check_word_chain_tc(bool clear);
 }  // namespace dqmc
 namespace {
 struct CheckUnit {
@@ -229,7 +230,7 @@ const CheckUnit kCheckUnits[] = {
     {"qrp_f64.cu", dqmc::check_word_qrp},     {"lu_f64.cu", dqmc::check_word_lu},
     {"jacobi_f64.cu", dqmc::check_word_jacobi}, {"chain_small.cu", dqmc::check_word_chain_small},
     {"ozaki_tc.cu", dqmc::check_word_ozaki}, {"gemm_tc.cu", dqmc::check_word_gemm_tc},
-    {"qrp_tc.cu", dqmc::check_word_qrp_tc},
+    {"qrp_tc.cu", dqmc::check_word_qrp_tc},   {"chain_tc.cu", dqmc::check_word_chain_tc},
 };
 #endif
 
@@ -403,6 +404,20 @@ inline int reduced_digits(dqmc_handle h, int N) {
   return h->prec == DQMC_CHAIN_BF16X8 && tc_wanted(h, N) ? 0 : (int)h->prec;
 }
 
+// Chunks of the FP64 chain in one tensor-core launch (chain_tc.cu): from N = 33,
+// the second K-block, up to the 128 rows of one MMA.  Equal-time chain, M = 100,
+// k = 10: N = 36 1 instance 1.78 -> 1.75 ms, 32 4.09 -> 3.62, 256 9.07 -> 6.06 ms;
+// N = 49 256 instances 16.3 -> 8.7 ms; N = 100 256 instances 25.2 -> 23.3.
+inline bool chain_tc_wanted(dqmc_handle h, int N) {
+  return !h->no_tc && N >= CHAIN_TC_MIN_N && N <= 128;
+}
+
+// The shared operand (the slice matrix), all that the fused chain needs.
+void take_tc_shared(Arena& ar, int N, TcWs& w) {
+  w.Es = ar.take<__nv_bfloat16>(tc_plane_elems(N, 128));   // either side (the left one is larger)
+  w.eEs = ar.take<int>(pad_to(N, 128));
+}
+
 void take_tc(Arena& ar, long long batch, int N, TcWs& w) {
   const long long ea = tc_plane_elems(N, 128), eb = tc_plane_elems(N, 64);
   long long cap = TC_SCRATCH / (2 * (ea + eb));
@@ -413,8 +428,7 @@ void take_tc(Arena& ar, long long batch, int N, TcWs& w) {
   w.B = ar.take<__nv_bfloat16>(w.cap * eb);
   w.eA = ar.take<int>((long long)w.cap * pad_to(N, 128));
   w.eB = ar.take<int>((long long)w.cap * pad_to(N, 64));
-  w.Es = ar.take<__nv_bfloat16>(ea);          // either side (ea >= eb)
-  w.eEs = ar.take<int>(pad_to(N, 128));
+  take_tc_shared(ar, N, w);
 }
 
 // Share q of nj of the digit slots, for products that run side by side (the
@@ -489,7 +503,7 @@ dqmc_status product(dqmc_handle h, int cls, double flops, const GemmArgs& g, con
 // Digits of a matrix all instances share, as the left or right operand.
 dqmc_status share_operand(dqmc_handle h, const double* X, int N, int R, int trans,
                           const TcWs& t) {
-  if (t.cap <= 0) return DQMC_OK;
+  if (!t.Es) return DQMC_OK;
   CK(tc_split(tc_operand(N, R, X, N, 0, trans, t.Es, t.eEs), 1, h->cur));
   return DQMC_OK;
 }
@@ -604,10 +618,11 @@ dqmc_status chunk_products(dqmc_handle h, int dir, int batch, int N, int M, int 
   long long sprev = s.instU;
   double* bufs[2] = {w.C0, w.C1};
   int nb = 0;
-  if (w.oz_s == 0 && w.tc.cap == 0 && N <= CHAIN_SMALL_MAX_N && batch <= 65535 &&
+  if (w.oz_s == 0 && (w.tc.Es ? chain_tc_wanted(h, N) : N <= CHAIN_SMALL_MAX_N && batch <= 65535) &&
       (dir > 0 || !lim)) {
     // small N: the whole chunk in one launch, each CTA applying every slice
-    // to a block of columns held in shared memory
+    // to a block of columns held in shared memory (on the tensor cores with E's
+    // digits, else on the FP64 pipe)
     ChainSmallArgs cs;
     cs.N = N; cs.batch = batch; cs.nslices = hi - lo + 1; cs.dir = dir; cs.lo = lo; cs.hi = hi;
     cs.E = E; cs.transE = dir < 0 ? 1 : 0;
@@ -615,7 +630,8 @@ dqmc_status chunk_products(dqmc_handle h, int dir, int batch, int N, int M, int 
     cs.C = w.C0; cs.sC = NN;
     cs.expV = expV; cs.sV = sV;
     cs.lim = lim; cs.lim_base = lo;
-    CKP(PC_CHAIN, 2.0 * N * N * (double)N * batch * (hi - lo + 1), chain_small(cs, st));
+    CKP(PC_CHAIN, 2.0 * N * N * (double)N * batch * (hi - lo + 1),
+        w.tc.Es ? chain_tc(cs, w.tc.Es, w.tc.eEs, status, 1, st) : chain_small(cs, st));
     *out = w.C0;
     return DQMC_OK;
   }
@@ -962,7 +978,7 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
   double* bufs[2] = {w.C0, w.C1};
   const double* prev = w.Iden;
   long long sprev = 0;
-  const bool small = N <= CHAIN_SMALL_MAX_N && Q <= 65535 && w.tc.cap == 0;
+  const bool small = w.tc.Es ? chain_tc_wanted(h, N) : N <= CHAIN_SMALL_MAX_N && Q <= 65535;
   CKS(share_operand(h, E, N, 128, 0, w.tc));
   if (small) {
     // small N: the k slices of every chunk in one launch (padding chunks copy
@@ -973,7 +989,8 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
     cs.C = bufs[0]; cs.sC = NN;
     cs.expV = expV; cs.sV = sV; cs.divS = P0; cs.sV_inner = (long long)k * N;
     cs.lim = w.len; cs.lim_base = 1;
-    CKP(PC_CHAIN, f2 * Q * k, chain_small(cs, st));
+    CKP(PC_CHAIN, f2 * Q * k,
+        w.tc.Es ? chain_tc(cs, w.tc.Es, w.tc.eEs, status, P0, st) : chain_small(cs, st));
     prev = bufs[0];
     sprev = NN;
   }
@@ -1579,6 +1596,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       tw.tc = TcWs{};
       tw.qr = QrWs{};
       if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, (long long)batch * tw.P0, N, tw.tc);
+      else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, tw.tc);
       if (tc && qrtc_wanted(h, N)) take_qr(ar, (long long)batch * tw.P0, N, 1, tw.qr);
       U = D = X0 = X1 = nullptr;
     } else {
@@ -1590,6 +1608,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       cw.tc = TcWs{};
       cw.qr = QrWs{};
       if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, batch, N, cw.tc);
+      else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, cw.tc);
       if (tc && qrtc_wanted(h, N)) take_qr(ar, batch, N, 0, cw.qr);
     }
     if (digits) take_ozaki(ar, batch, N, digits, cw);
@@ -2179,6 +2198,9 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       // the first also serves the products over all stack slots after the chains
       take_tc(ar, Q, N, cw.tc);
       take_tc(ar, batch, N, cw2.tc);
+    } else if (tc && !reduced_digits(h, N) && chain_tc_wanted(h, N)) {
+      take_tc_shared(ar, N, cw.tc);
+      take_tc_shared(ar, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
       take_qr(ar, Q, N, 0, cw.qr);
@@ -2241,7 +2263,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
     const double f2 = 2.0 * N * (double)N * N * Q;
     // E is still the shared left operand of cw.tc; E^{-1} becomes the shared
     // right operand in the backward chain's slot
-    CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
+    if (cw.tc.cap > 0) CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
     TcWs wr = cw.tc;
     wr.Es = cw2.tc.Es; wr.eEs = cw2.tc.eEs;
     for (int s = 0; s < k; ++s) {
@@ -2344,6 +2366,9 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       // the first also serves the products over all stack slots after the chains
       take_tc(ar, Q, N, cw.tc);
       take_tc(ar, batch, N, cw2.tc);
+    } else if (tc && !reduced_digits(h, N) && chain_tc_wanted(h, N)) {
+      take_tc_shared(ar, N, cw.tc);
+      take_tc_shared(ar, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
       take_qr(ar, Q, N, 0, cw.qr);
@@ -2393,7 +2418,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
               sw.XF + nc * NN, nt * NN, nullptr, ldo, sgo, stout, lw, cw.qr));
   // checkpoints G_{jk+1}
   CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, Gw, nullptr, nullptr, stout, cw.tc, cw.qr));
-  CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
+  if (cw.tc.cap > 0) CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
   TcWs wr = cw.tc;                                     // E^{-1} as the shared right operand
   wr.Es = cw2.tc.Es; wr.eEs = cw2.tc.eEs;
   const double wflops = 2.0 * N * (double)N * N * Q;
@@ -2531,6 +2556,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       w.cw.qr = QrWs{};
       const int digits = reduced_digits(h, N);
       if (tc && !digits && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
+      else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, w.cw.tc);
       if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr);
       if (digits) take_ozaki(ar, nb, N, digits, w.cw);
       take_loh(ar, nb, N, w.lw);

@@ -340,6 +340,12 @@ struct TcGemmArgs {
   const double* csrc = nullptr; long long scsrc = 0, ldcsrc = 0;
 };
 cudaError_t tc_gemm(const TcGemmArgs& a, int batch, cudaStream_t st);
+
+// chain_small's products on the tensor cores (chain_tc.cu), Es and eEs the
+// digits of E (of E^T backward) as a left operand.
+constexpr int CHAIN_TC_MIN_N = 33;
+cudaError_t chain_tc(const ChainSmallArgs& c, const __nv_bfloat16* Es, const int* eEs, int* status,
+                     int status_div, cudaStream_t st);
 }  // namespace dqmc
 
 // ---------------------------------------------------------------------------
