@@ -443,14 +443,22 @@ TcWs tc_part(const TcWs& w, int q, int nj, int N) {
   return p;
 }
 
-// Left (R = 128: rows of op(X)) or right (R = 64: columns of op(X)) operand of
-// an N x N product; one instance when sX == 0.
-TcSplitArgs tc_operand(int N, int R, const double* X, long long ld, long long sX, int trans,
-                       __nv_bfloat16* S, int* e) {
+// Whether a product with a shared operand stacks the other one's instances, 32
+// rows of one filling up the 128-row tile of another, instead of padding each to
+// whole tiles: where that saves an eighth of the rows.  The gradient of 64
+// instances at N = 144 (160 instead of 256 rows) 94.7 -> 80.1 ms; with no less
+// rows the stacked launch is the slower one: equal-time chain, N = 256, 128
+// instances 111.6 -> 112.1 ms, N = 324 (352 of 384 rows), 20.3 -> 20.7 ms.
+inline bool stack_wanted(int N) { return 8 * pad_to(N, 32) <= 7 * pad_to(N, 128); }
+
+// Rows (rows = true) or columns of op(X) as digit tiles of R = 128 (left operand
+// of a product) or 64 (right); one instance when sX == 0.
+TcSplitArgs tc_operand(int N, int R, bool rows, const double* X, long long ld, long long sX,
+                       int trans, __nv_bfloat16* S, int* e) {
   TcSplitArgs a;
   a.X = X; a.sX = sX;
-  // left: element (k, row) of op(X) is X[row ld + k]; right: (k, col) is X[k ld + col]
-  const bool along_k = (R == 128) != (trans != 0);
+  // element (k, row) of op(X) is X[row ld + k], (k, col) is X[k ld + col]
+  const bool along_k = rows != (trans != 0);
   a.ldm = along_k ? 1 : ld;
   a.ldj = along_k ? ld : 1;
   a.N = N; a.R = R; a.PJ = pad_to(N, R); a.PM = pad_to(N, 32);
@@ -461,33 +469,43 @@ TcSplitArgs tc_operand(int N, int R, const double* X, long long ld, long long sX
 
 // One batched N x N product of the method: on the tensor cores when t has
 // room, else on the FP64 pipe.  shared_A / shared_B: t.Es already holds that
-// operand's digits.  A diagonal ms between the operands goes to the
+// operand's digits; where the other one's are stacked as the left operand, E X_b
+// is the transpose of X_b^T E^T.  A diagonal ms between the operands goes to the
 // per-instance one.
 dqmc_status product(dqmc_handle h, int cls, double flops, const GemmArgs& g, const TcWs& t,
                     int* status, int status_div = 1, bool shared_A = false,
                     bool shared_B = false) {
   if (t.cap <= 0 || g.cs || g.addIdentity || g.alpha_ptr || g.skip_if || g.divA != 1 ||
-      g.divB != 1 || g.divC != 1 || (shared_A && shared_B)) {
+      g.divB != 1 || g.divC != 1 || (shared_A && shared_B) || (shared_B && g.lim)) {
     CKP(cls, flops, gemm_f64(g, h->cur));
     return DQMC_OK;
   }
   const int N = g.N;
-  TcSplitArgs sa = tc_operand(N, 128, g.A, g.lda, g.sA, g.transA, t.A, t.eA);
-  TcSplitArgs sb = tc_operand(N, 64, g.B, g.ldb, g.sB, g.transB, t.B, t.eB);
-  sb.gm = g.permB; sb.sgm = g.sperm;
-  TcSplitArgs& sm = shared_B ? sa : sb;
+  const int stack = !stack_wanted(N) ? 0 : (shared_A ? 2 : (shared_B ? 1 : 0));
+  // left and right operand of the launch (without the shared one)
+  TcSplitArgs sa = stack == 2 ? tc_operand(N, 128, false, g.B, g.ldb, g.sB, g.transB, t.A, t.eA)
+                            : tc_operand(N, 128, true, g.A, g.lda, g.sA, g.transA, t.A, t.eA);
+  TcSplitArgs sb = tc_operand(N, 64, false, g.B, g.ldb, g.sB, g.transB, t.B, t.eB);
+  (stack == 2 ? sa : sb).gm = g.permB; (stack == 2 ? sa : sb).sgm = g.sperm;
+  if (stack) {
+    sa.stack = 1;
+    sa.PJ = pad_to(N, 32); sa.se = sa.PJ;
+  }
+  const bool own_a = stack || !shared_A, own_b = !stack && !shared_B;
+  TcSplitArgs& sm = own_b ? sb : sa;
   sm.sc = g.ms; sm.ssc = g.sms; sm.ssc_inner = g.sms_inner; sm.divS = g.divS;
   sa.lim = sb.lim = g.lim; sa.lim_at = sb.lim_at = g.lim_at;
   for (int b0 = 0; b0 < g.batch; b0 += t.cap) {
     const int nb = g.batch - b0 < t.cap ? g.batch - b0 : t.cap;
     sa.b0 = sb.b0 = b0;
-    if (!shared_A) CK(tc_split(sa, nb, h->cur));
-    if (!shared_B) CK(tc_split(sb, nb, h->cur));
+    if (own_a) CK(tc_split(sa, nb, h->cur));
+    if (own_b) CK(tc_split(sb, nb, h->cur));
     TcGemmArgs m;
-    m.A = shared_A ? t.Es : t.A; m.eA = shared_A ? t.eEs : t.eA;
-    m.sA = shared_A ? 0 : sa.sS; m.seA = shared_A ? 0 : sa.se;
-    m.B = shared_B ? t.Es : t.B; m.eB = shared_B ? t.eEs : t.eB;
-    m.sB = shared_B ? 0 : sb.sS; m.seB = shared_B ? 0 : sb.se;
+    m.A = own_a ? t.A : t.Es; m.eA = own_a ? t.eA : t.eEs;
+    m.sA = own_a ? sa.sS : 0; m.seA = own_a ? sa.se : 0;
+    m.B = own_b ? t.B : t.Es; m.eB = own_b ? t.eB : t.eEs;
+    m.sB = own_b ? sb.sS : 0; m.seB = own_b ? sb.se : 0;
+    m.stack = stack;
     m.N = N; m.nkb = sa.PM / 32; m.upperA = g.upperA; m.b0 = b0;
     m.C = g.C; m.ldc = g.ldc; m.sC = g.sC;
     m.scaled = g.rs || g.alpha != 1.0; m.alpha = g.alpha;
@@ -500,12 +518,23 @@ dqmc_status product(dqmc_handle h, int cls, double flops, const GemmArgs& g, con
   return DQMC_OK;
 }
 
-// Digits of a matrix all instances share, as the left or right operand.
-dqmc_status share_operand(dqmc_handle h, const double* X, int N, int R, int trans,
+// Digits of a matrix all instances share, as rows or columns of op(X) in tiles of R.
+dqmc_status share_operand(dqmc_handle h, const double* X, int N, int R, bool rows, int trans,
                           const TcWs& t) {
   if (!t.Es) return DQMC_OK;
-  CK(tc_split(tc_operand(N, R, X, N, 0, trans, t.Es, t.eEs), 1, h->cur));
+  CK(tc_split(tc_operand(N, R, rows, X, N, 0, trans, t.Es, t.eEs), 1, h->cur));
   return DQMC_OK;
+}
+
+// op(X) as the shared left operand of product().
+dqmc_status share_left(dqmc_handle h, const double* X, int N, int trans, const TcWs& t) {
+  return share_operand(h, X, N, stack_wanted(N) ? 64 : 128, true, trans, t);
+}
+
+// The slice matrix (its transpose for the backward chain) for the chain's products.
+dqmc_status share_slice(dqmc_handle h, const double* E, int N, int trans, const TcWs& t) {
+  return chain_tc_wanted(h, N) ? share_operand(h, E, N, 128, true, trans, t)
+                               : share_left(h, E, N, trans, t);
 }
 
 // Slots of the blocked pivoted QR (qrp_tc.cu); without slots the factorisation
@@ -674,7 +703,8 @@ dqmc_status chunk_products(dqmc_handle h, int dir, int batch, int N, int M, int 
       g.transA = 1;                                          // diag(e^{V_l}) E^T A
       g.rs = expV + (long long)(l - 1) * N; g.srs = sV;
     }
-    CKS(product(h, PC_CHAIN, 2.0 * N * N * (double)N * batch, g, w.tc, status, 1, true));
+    CKS(product(h, PC_CHAIN, 2.0 * N * N * (double)N * batch, g, w.tc, status, 1,
+                !chain_tc_wanted(h, N)));
     prev = bufs[nb];
     sprev = NN;
     nb ^= 1;
@@ -979,7 +1009,7 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
   const double* prev = w.Iden;
   long long sprev = 0;
   const bool small = w.tc.Es ? chain_tc_wanted(h, N) : N <= CHAIN_SMALL_MAX_N && Q <= 65535;
-  CKS(share_operand(h, E, N, 128, 0, w.tc));
+  CKS(share_slice(h, E, N, 0, w.tc));
   if (small) {
     // small N: the k slices of every chunk in one launch (padding chunks copy
     // the identity through)
@@ -1661,7 +1691,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
     CKS(run_inversion(h, batch, N, Ut, NN, Dt, N, Xt, NN, Gout, ldout, sgout, stout, lw, pw, tw.qr));
   } else {
     if (cw.oz_s > 0) CK(split_E(E, N, 0, cw, st));   // E slices, shared by all instances
-    CKS(share_operand(h, E, N, 128, 0, cw.tc));
+    CKS(share_slice(h, E, N, 0, cw.tc));
     CK(set_identity(U, NN, N, batch, st));
     CK(set_const(D, (long long)N * batch, 1.0, st));
     CK(set_identity(X0, NN, N, batch, st));
@@ -1869,8 +1899,8 @@ dqmc_status run_stacks(dqmc_handle h, int batch, int N, int M, int k, const doub
     CK(split_E(E, N, 0, cw, st));
     CK(split_E(E, N, 1, cw2, st));
   }
-  CKS(share_operand(h, E, N, 128, 0, cw.tc));
-  CKS(share_operand(h, E, N, 128, 1, cw2.tc));
+  CKS(share_slice(h, E, N, 0, cw.tc));
+  CKS(share_slice(h, E, N, 1, cw2.tc));
   CK(set_identity(w.UF, nt * NN, N, batch, st));
   CK(set_const_strided(w.DF, (long long)nt * N, N, batch, 1.0, st));
   CK(set_identity(w.XF, nt * NN, N, batch, st));
@@ -2261,9 +2291,11 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
     if (expmV) CK(exp_pad(Vd, expmV, batch, M, (int)Mp, N, -1.0, nullptr, st, sh));
     double* dst[3] = {Gtto, Gt0o, G0to};
     const double f2 = 2.0 * N * (double)N * N * Q;
-    // E is still the shared left operand of cw.tc; E^{-1} becomes the shared
-    // right operand in the backward chain's slot
-    if (cw.tc.cap > 0) CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
+    // E shared in the forward chain's slot, E^{-1} in the backward chain's
+    if (cw.tc.cap > 0) {
+      CKS(share_left(h, ew.t0, N, 0, cw.tc));
+      CKS(share_operand(h, ewi.t0, N, 64, false, 0, cw2.tc));
+    }
     TcWs wr = cw.tc;
     wr.Es = cw2.tc.Es; wr.eEs = cw2.tc.eEs;
     for (int s = 0; s < k; ++s) {
@@ -2418,7 +2450,10 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
               sw.XF + nc * NN, nt * NN, nullptr, ldo, sgo, stout, lw, cw.qr));
   // checkpoints G_{jk+1}
   CKS(run_two_stack_inversion(h, (int)Q, N, nt, sw, mw, Gw, nullptr, nullptr, stout, cw.tc, cw.qr));
-  if (cw.tc.cap > 0) CKS(share_operand(h, ewi.t0, N, 64, 0, cw2.tc));
+  if (cw.tc.cap > 0) {
+    CKS(share_left(h, ew.t0, N, 0, cw.tc));
+    CKS(share_operand(h, ewi.t0, N, 64, false, 0, cw2.tc));
+  }
   TcWs wr = cw.tc;                                     // E^{-1} as the shared right operand
   wr.Es = cw2.tc.Es; wr.eEs = cw2.tc.eEs;
   const double wflops = 2.0 * N * (double)N * N * Q;
@@ -2666,7 +2701,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
         if (!E_pool) CKS(run_expm(h, K_pool + g.offK, N, g.dtau, -1.0, w.ew, w.st, nb));
         CK(exp_gather(V_pool, w.offV, w.Mb, nb, (int)Mp, N, w.expV, w.st, st));
         if (w.cw.oz_s > 0) CK(split_E(E, N, 0, w.cw, st));   // E slices, shared by the group
-        CKS(share_operand(h, E, N, 128, 0, w.cw.tc));
+        CKS(share_slice(h, E, N, 0, w.cw.tc));
         CK(set_identity(w.U, NN, N, nb, st));
         CK(set_const(w.D, (long long)N * nb, 1.0, st));
         CK(set_identity(w.X0, NN, N, nb, st));

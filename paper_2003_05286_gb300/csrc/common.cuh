@@ -320,18 +320,21 @@ struct TcSplitArgs {
   const int* gm = nullptr; long long sgm = 0;
   int N = 0, PJ = 0, PM = 0, R = 64;
   int upper = 0;                                 // entries with m < j count as zero
+  int stack = 0;                                 // all instances' rows in one run of tiles
   __nv_bfloat16* S = nullptr; long long sS = 0;
   int* e = nullptr; long long se = 0;
   int b0 = 0;                                    // instance of slot 0
   const int* lim = nullptr; int lim_at = 0;      // ended instances are left out
 };
 cudaError_t tc_split(const TcSplitArgs& a, int batch, cudaStream_t st);
-// C_b = alpha diag(rs_b) A_b B_b for the operand slots 0 .. batch - 1 holding
+// C_b = alpha diag(rs_b) A_b B_b (stack 2: its transpose, rs_b on C's rows) for the operand slots 0 .. batch - 1 holding
 // instances b0 + slot; instances with lim[b] < lim_at copy csrc_b instead.
 struct TcGemmArgs {
   const __nv_bfloat16* A = nullptr; const int* eA = nullptr; long long sA = 0, seA = 0;
   const __nv_bfloat16* B = nullptr; const int* eB = nullptr; long long sB = 0, seB = 0;
   int N = 0, nkb = 0, upperA = 0, b0 = 0;
+  int stack = 0;                                 // 1, 2: stacked left operands (gemm_tc.cu)
+  int slots = 0, groups = 0;                     // set by tc_gemm
   double* C = nullptr; long long ldc = 0, sC = 0;
   int scaled = 0; double alpha = 1.0;            // scaled: alpha and rs apply
   const double* rs = nullptr; long long srs = 0; int divS = 1;

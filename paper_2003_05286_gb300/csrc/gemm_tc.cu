@@ -38,6 +38,8 @@
 // digits of a tile.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -75,7 +77,13 @@ constexpr uint32_t TC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) 
 // one another and run at a third of the rate.  Shared-memory bandwidth bounds
 // the loop (12 KB read per 128-cycle MMA, 96 KB copied per 24 of them).
 // WIN: 1 when K <= 128 (no drain), 2 when K <= 256 (block 1 drains once), 3 else.
-template <int WIN>
+// STACK: the left operands of all instances form one tall matrix, whose 32-row
+// groups (one per epilogue warp) fill the tiles; the right operand is shared.
+// 1: C_b = A_b B, 2: C_b = (A_b B)^T, for products whose shared operand is the left one.
+// At N = 144 an instance then takes 160 rows of tiles instead of 256, 3.75 tiles
+// instead of 6, and K stops at the last 16 values that hold any: the wraps of a
+// gradient of 64 instances (1344 checkpoints) and its chains 94.7 -> 80.1 ms.
+template <int WIN, int STACK>
 __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
@@ -89,7 +97,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n0 = blockIdx.x * TC_BN, m0 = blockIdx.y * TC_BM;
-  const int z = blockIdx.z;            // operand slot
+  const int z = STACK ? 0 : blockIdx.z;   // operand slot
   const int b = a.b0 + z;              // instance
   const int N = a.N;
   const int kb0 = a.upperA ? m0 / TC_BK : 0, nk = a.nkb - kb0;
@@ -102,7 +110,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
     return;
   // an instance whose chain has ended: its source passes through (uniform over
   // the CTA, before any barrier or TMEM allocation)
-  if (a.lim && a.lim[b] < a.lim_at) {
+  if (!STACK && a.lim && a.lim[b] < a.lim_at) {
     const double* src = a.csrc + (long long)b * a.scsrc;
     double* dst = a.C + (long long)b * a.sC;
     for (int e = tid; e < TC_BM * TC_BN; e += TC_THREADS) {
@@ -189,7 +197,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          for (int kk = 0; kk < TC_BK / 16; ++kk) {
+          const int nkk = (kb0 + i) * TC_BK + 16 < N ? 2 : 1;   // all k beyond are zero
+          for (int kk = 0; kk < nkk; ++kk) {
             const uint64_t dAk = dA + (uint64_t)(kk * 2), dBk = dB + (uint64_t)(kk * 2);
             for (int p = 0; p <= 4 * r + 3; ++p)
               umma(tmem + (uint32_t)(256 * r), dAk + (uint64_t)(p * (TC_A_TILE >> 4)),
@@ -210,7 +219,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
     // ---- epilogue ------------------------------------------------------------
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const int cbase = (warp >> 2) * 16;
-    const int rl = (warp & 3) * 32 + lane, row = m0 + rl;
+    const int rl = (warp & 3) * 32 + lane;
+    const int grp = 4 * blockIdx.y + (warp & 3);         // 32-row group of the stack
+    const int zs = STACK ? grp / a.groups : z;
+    const int row = STACK ? (grp - zs * a.groups) * 32 + lane : m0 + rl;
     const int nwin = (nk + 3) / 4;             // windows of block 1 (block 0: every second)
     long long lo[WIN >= 2 ? 16 : 1], hi[WIN >= 3 ? 16 : 1];
     bool ok = true;
@@ -269,10 +281,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
     ok = *(volatile int*)s_fail == 0;          // uniform over the epilogue warps
     if (ok) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int ea = row < N ? a.eA[(long long)z * a.seA + row] : 0;
+      const int bs = a.b0 + zs;
+      const bool have = row < N && zs < a.slots;
+      const int ea = have ? a.eA[(long long)zs * a.seA + row] : 0;
+      const bool ended = STACK == 2 && have && a.lim && a.lim[bs] < a.lim_at;
       const int* eB = a.eB + (long long)z * a.seB;
       double rscale = a.alpha;
-      if (a.rs && row < N) rscale *= a.rs[(long long)(b / a.divS) * a.srs + row];
+      if (STACK != 2 && a.rs && have) rscale *= a.rs[(long long)(bs / a.divS) * a.srs + row];
+      const double* crs = STACK == 2 && a.rs && have ? a.rs + (long long)(bs / a.divS) * a.srs : nullptr;
+      double* cst = a.C + (long long)bs * a.sC + row;
+      const double* cend = ended ? a.csrc + (long long)bs * a.scsrc + row : nullptr;
       double* ctile = reinterpret_cast<double*>(base);   // the stages are idle now
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -300,21 +318,32 @@ __global__ void __launch_bounds__(TC_THREADS, 1) tc_gemm_kernel(const TcGemmArgs
           double v = split_times_pow2(h + (l >> 32), (unsigned int)(l & 0xFFFFFFFFll),
                                       ea + eb - 8 * (TC_S + 1));
           if (ea >= TC_NONFINITE || eb >= TC_NONFINITE) v = __longlong_as_double(0x7ff8000000000000ll);
-          ctile[rl * TC_C_LD + cbase + 8 * c + j] = v;
+          if (STACK == 2) {                      // lanes along the rows of C
+            if (have && col < N) {
+              if (a.scaled) v *= crs ? rscale * crs[col] : rscale;
+              cst[(long long)col * a.ldc] = ended ? cend[(long long)col * a.ldcsrc] : v;
+            }
+          } else {
+            ctile[rl * TC_C_LD + cbase + 8 * c + j] = v;
+          }
         }
       }
-      if (a.scaled) {   // row scale (and alpha): one FP64 multiply per entry
+      if (STACK != 2 && a.scaled) {   // row scale (and alpha): one FP64 multiply per entry
 #pragma unroll 4
         for (int j = 0; j < 16; ++j) ctile[rl * TC_C_LD + cbase + j] *= rscale;
       }
-      asm volatile("bar.sync 1, %0;" ::"r"(TC_EPI) : "memory");
-      double* Cb = a.C + (long long)b * a.sC;
-      for (int e = tid; e < TC_BM * TC_BN; e += TC_EPI) {
-        const int r = e / TC_BN, c = e % TC_BN;
-        if (m0 + r < N && n0 + c < N) Cb[(long long)(m0 + r) * a.ldc + n0 + c] = ctile[r * TC_C_LD + c];
+      if (STACK != 2) {
+        asm volatile("bar.sync 1, %0;" ::"r"(TC_EPI) : "memory");
+        for (int e = tid; e < TC_BM * TC_BN; e += TC_EPI) {
+          const int r = e / TC_BN, c = e % TC_BN;
+          const int g = 4 * blockIdx.y + (r >> 5), zr = STACK ? g / a.groups : z;
+          const int cr = STACK ? (g - zr * a.groups) * 32 + (r & 31) : m0 + r;
+          if (zr < a.slots && cr < N && n0 + c < N)
+            a.C[(long long)(a.b0 + zr) * a.sC + (long long)cr * a.ldc + n0 + c] = ctile[r * TC_C_LD + c];
+        }
       }
-    } else if (tid == 0 && a.status) {
-      atomicOr(&a.status[b / a.status_div], DQMC_STATUS_TIMEOUT);
+    } else if (a.status && (STACK ? lane == 0 && warp < 4 && zs < a.slots : tid == 0)) {
+      atomicOr(&a.status[(a.b0 + zs) / a.status_div], DQMC_STATUS_TIMEOUT);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
@@ -411,15 +440,16 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const TcSplitArgs a) {
     a.e[(long long)z * a.se + j0 + tid] = e;
   }
   __syncthreads();
-  __nv_bfloat16* S = a.S + (long long)z * a.sS;
+  __nv_bfloat16* S = a.S + (a.stack ? 0 : (long long)z * a.sS);
+  const int jt = (a.stack ? z * a.PJ : 0) + j0;   // the CTA's first row of the stack
   const int ch = tid & 3, nkb = PM / 32;
   const int plane = a.R * 32;
   for (int it = tid >> 2; it < 32 * nkb; it += 64) {
     const int jj = it & 31, kb = it >> 5;
     const int e = emax[0][jj];
     const int mb = kb * 32 + ch * 8;
-    const int jr = (j0 + jj) % a.R;
-    __nv_bfloat16* out = S + ((long long)((j0 + jj) / a.R) * nkb + kb) * (TC_S * (long long)plane) +
+    const int jr = (jt + jj) % a.R;
+    __nv_bfloat16* out = S + ((long long)((jt + jj) / a.R) * nkb + kb) * (TC_S * (long long)plane) +
                          jr * 32 + ((ch ^ ((jr >> 1) & 3)) << 3);   // 64-byte swizzle
     tc_digits8(e, [&](int k) { return tile[(mb + k) * 33 + jj]; }, [&](int q, uint4 w) {
       if (DQMC_CHECK((reinterpret_cast<uintptr_t>(out + q * plane) & 15) == 0, q))
@@ -430,7 +460,7 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const TcSplitArgs a) {
 
 cudaError_t tc_split(const TcSplitArgs& a, int batch, cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
-  if (batch > 65535 || a.PM % 32 || a.PJ % a.R || a.R % 32 || a.PM < a.N || a.PJ < a.N ||
+  if (batch > 65535 || a.PM % 32 || a.PJ % (a.stack ? 32 : a.R) || a.R % 32 || a.PM < a.N || a.PJ < a.N ||
       a.sS % 8 || (reinterpret_cast<uintptr_t>(a.S) & 15) || (a.ldm != 1 && a.ldj != 1))
     return cudaErrorInvalidValue;
   const size_t sm = (size_t)a.PM * 33 * sizeof(double);
@@ -446,20 +476,32 @@ cudaError_t tc_split(const TcSplitArgs& a, int batch, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t tc_gemm(const TcGemmArgs& a, int batch, cudaStream_t st) {
+cudaError_t tc_gemm(const TcGemmArgs& args, int batch, cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
-  if (batch > 65535 || a.nkb < 1 || a.nkb * TC_BK < a.N || a.N > TC_MAX_N || (a.lim && !a.csrc))
+  TcGemmArgs a = args;
+  if (batch > 65535 || a.nkb < 1 || a.nkb * TC_BK < a.N || a.N > TC_MAX_N || (a.lim && !a.csrc) ||
+      (a.stack && (a.upperA || a.sB != 0)) || (a.stack == 1 && a.lim))
     return cudaErrorInvalidValue;
-  const dim3 grid((a.N + TC_BN - 1) / TC_BN, (a.N + TC_BM - 1) / TC_BM, batch);
+  a.slots = batch;
+  a.groups = (a.N + 31) / 32;
+  const long long rows = a.stack ? ((long long)batch * a.groups + 3) / 4 : (a.N + TC_BM - 1) / TC_BM;
+  if (rows > 65535) return cudaErrorInvalidValue;
+  const dim3 grid((a.N + TC_BN - 1) / TC_BN, (int)rows, a.stack ? 1 : batch);
   auto go = [&](auto kern) {
     const cudaError_t e = allow_dyn_smem(kern);
     if (e != cudaSuccess) return e;
     kern<<<grid, TC_THREADS, TC_SMEM, st>>>(a);
     return cudaGetLastError();
   };
-  if (a.nkb <= 4) return go(tc_gemm_kernel<1>);
-  if (a.nkb <= 8) return go(tc_gemm_kernel<2>);
-  return go(tc_gemm_kernel<3>);
+  auto pick = [&](auto win) {
+    constexpr int W = decltype(win)::value;
+    if (a.stack == 1) return go(tc_gemm_kernel<W, 1>);
+    if (a.stack == 2) return go(tc_gemm_kernel<W, 2>);
+    return go(tc_gemm_kernel<W, 0>);
+  };
+  if (a.nkb <= 4) return pick(std::integral_constant<int, 1>{});
+  if (a.nkb <= 8) return pick(std::integral_constant<int, 2>{});
+  return pick(std::integral_constant<int, 3>{});
 }
 
 }  // namespace dqmc
