@@ -78,8 +78,8 @@ enum dqmc_status_bits {
  * scales), the digit products accumulate exactly in FP32 on the tcgen05
  * tensor cores and are recombined in FP64; a product is accurate to about
  * N 2^{-7s-1} of (row max x column max), normwise rather than elementwise.
- * From N = 64 the FP64 products themselves run on the tensor cores (eight
- * base-256 digits, about N 2^{-58}), and DQMC_CHAIN_BF16X8 uses them.
+ * The FP64 products themselves run on the tensor cores from N = 33 (eight
+ * base-256 digits, about N 2^{-58}), and DQMC_CHAIN_BF16X8 uses the FP64 chain.
  * Supported for N <= 256 in dqmc_greens, dqmc_logdet, dqmc_greens_tdisplaced,
  * dqmc_logdet_grad (both stacks) and dqmc_greens_ragged (every instance N <= 256);
  * N > 256 returns DQMC_ERR_UNSUPPORTED (dqmc_greens_noalloc takes no handle
@@ -126,9 +126,9 @@ dqmc_status dqmc_set_graph_mode(dqmc_handle h, int enable);
  * (paper_2003_05286_gb300/tune.py); results do not depend on it. */
 dqmc_status dqmc_set_gemm_tile(dqmc_handle h, int tile);
 
-/* How the equal-time chain of dqmc_greens / dqmc_logdet is folded (FP64
- * chain precision only; the other calls and the mixed precisions always run
- * the sequential chain):
+/* How the equal-time chain of dqmc_greens / dqmc_logdet is folded (chain
+ * precisions FP64 and BF16X8; the other calls and precisions always run the
+ * sequential chain):
  *   DQMC_FOLD_SEQUENTIAL  chunk after chunk, Eq. (stabmult) with the running
  *                         U D X (one pivoted QR per chunk, in order);
  *   DQMC_FOLD_TREE        all chunk products at once, each decomposed, then

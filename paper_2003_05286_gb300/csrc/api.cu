@@ -396,12 +396,16 @@ inline bool tc_wanted(dqmc_handle h, int N) {
 
 // Digits of the reduced-precision chain (ozaki_tc.cu), 0 for products in FP64
 // accuracy.  Eight BF16 digits per operand are what the FP64 products take too,
-// with 8 instead of 7 bits each: DQMC_CHAIN_BF16X8 runs on them wherever they
-// serve (one product of 128 instances, N = 256: 218 -> 170 us, its split 79 ->
-// 43, error 2^-58 instead of 2^-51 of row max x column max).
+// with 8 instead of 7 bits each, and below N = 33 the FP64 pipe needs less time
+// than any digits: DQMC_CHAIN_BF16X8 runs on the FP64 chain.  One product of 128
+// instances, N = 256: 218 -> 170 us, its split 79 -> 43, error 2^-58 instead of
+// 2^-51 of row max x column max.  Equal-time chain, M = 100, k = 5: N = 9, 64
+// instances 4.69 -> 0.99 ms, N = 25, 256 instances 8.94 -> 4.43, N = 36, 256
+// instances 12.6 -> 9.4; one instance (tree fold) N = 256 39.9 -> 15.7.  Only a call that had no room for the tensor cores'
+// scratch under capture (no_tc) still takes the base-128 digits.
 inline int reduced_digits(dqmc_handle h, int N) {
   if (h->prec == DQMC_CHAIN_FP64) return 0;
-  return h->prec == DQMC_CHAIN_BF16X8 && tc_wanted(h, N) ? 0 : (int)h->prec;
+  return h->prec == DQMC_CHAIN_BF16X8 && (!h->no_tc || N < CHAIN_TC_MIN_N) ? 0 : (int)h->prec;
 }
 
 // Chunks of the FP64 chain in one tensor-core launch (chain_tc.cu): from N = 33,
@@ -1123,8 +1127,8 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
 // Tree fold for the equal-time chain: by setting, or (auto) when the level-0
 // QRs of all chunks of the batch fit in one wave of CTAs (one per SM) and the
 // chain has at least four chunks.
-bool use_tree(dqmc_handle h, int batch, int nc) {
-  if (h->prec != DQMC_CHAIN_FP64 || h->decomp != DQMC_DECOMP_QR) return false;
+bool use_tree(dqmc_handle h, int batch, int N, int nc) {
+  if (reduced_digits(h, N) != 0 || h->decomp != DQMC_DECOMP_QR) return false;
   if (h->fold == DQMC_FOLD_TREE) return nc > 1;
   if (h->fold == DQMC_FOLD_SEQUENTIAL) return false;
   return nc >= 4 && (long long)batch * nc <= h->sms;
@@ -1604,7 +1608,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   const bool host = h->pmode == DQMC_PTR_HOST;
   const long long NN = (long long)N * N;
   const int nc = n_chunks(M, k);
-  const bool tree = use_tree(h, batch, nc);
+  const bool tree = use_tree(h, batch, N, nc);
   // padded slice stride of exp(V): one spare chunk, and for the tree every
   // padding chunk of its power-of-two width
   const int mp_chunks = tree && tree_width(nc) > nc + 1 ? tree_width(nc) : nc + 1;
