@@ -401,8 +401,9 @@ inline bool tc_wanted(dqmc_handle h, int N) {
 // instances, N = 256: 218 -> 170 us, its split 79 -> 43, error 2^-58 instead of
 // 2^-51 of row max x column max.  Equal-time chain, M = 100, k = 5: N = 9, 64
 // instances 4.69 -> 0.99 ms, N = 25, 256 instances 8.94 -> 4.43, N = 36, 256
-// instances 12.6 -> 9.4; one instance (tree fold) N = 256 39.9 -> 15.7.  Only a call that had no room for the tensor cores'
-// scratch under capture (no_tc) still takes the base-128 digits.
+// instances 12.6 -> 9.4; one instance (tree fold) N = 256 39.9 -> 15.7.  Only a
+// call that had no room for the tensor cores' scratch under capture (no_tc) still
+// takes the base-128 digits.
 inline int reduced_digits(dqmc_handle h, int N) {
   if (h->prec == DQMC_CHAIN_FP64) return 0;
   return h->prec == DQMC_CHAIN_BF16X8 && (!h->no_tc || N < CHAIN_TC_MIN_N) ? 0 : (int)h->prec;

@@ -1,5 +1,6 @@
 // The k slice products of one chunk in one launch, for N <= 128 (Sec. 2,
-// Eq. (Ztr); the naive products between two re-factorisations, Sec. 4.1).
+// Eq. (Ztr); the naive products between two re-factorisations, Sec. 4.1): for N < 33,
+// and above where there is no room for chain_tc.cu's digits.
 //
 // Forward chain:  C <- E diag(e^{V_l}) C   for l = lo .. hi
 // Backward chain: C <- diag(e^{V_l}) E^T C for l = hi .. lo   (B_l^T, App. A)

@@ -63,6 +63,8 @@ constexpr int RING = 4 * VT_TILE;         // staging of both kernels (64 KB)
 constexpr int TLD = 33;
 constexpr int QF = 2 * 8 * 52;             // floats of two staged FP32 columns (8 x 52 >= 4 x 68)
 constexpr int XS = QRTC_MAX_N;            // rows of a staged FP64 column
+enum { QP_SMALL, QP_MID, QP_BIG };        // forms of the panel kernel
+__host__ __device__ constexpr int xs_rows(bool small) { return small ? 64 : XS; }
 // BF16 operands (K-major), FP32 accumulator, M = 128, N = 128
 constexpr uint32_t IDESC_128 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) |
                                ((128u >> 4) << 24);
@@ -125,7 +127,7 @@ __device__ __forceinline__ int row_rho(const double* Drow, int r, int N) {
 // Bound by shared-memory reads of the pivot column and FP32 issue; two columns
 // per thread, which halve those reads, took twice as long (263 against 125
 // thousand cycles for 32 steps of 256 rows).
-template <int TPC, int KM, bool GR>
+template <int TPC, int KM, bool GR, bool SMALL>
 __device__ __noinline__ void pivot_search(const double* W, const double* Din, const float* lnrm,
                                           const int* s_rem, const int* s_cand, int N, int j0,
                                           int m, int nb, float* qf, float* s_inv,
@@ -292,9 +294,9 @@ __device__ __forceinline__ void norm_and_gamma(double sig, double alpha, double&
 // holds its sub-partition's pipe for 64 cycles: short panels take 8 lanes (few
 // reduction levels, few warps), tall ones 16 (the columns left spread evenly
 // over the sub-partitions; N = 256, 32 columns: 323 -> 240 thousand cycles).  A
-// warp whose columns are done drops out.  Leaves R in W^T and u_j (zeros above j) in out[0]; out[1]: two columns
-// of workspace.
-template <int LPC, int KR>
+// warp whose columns are done drops out.  Leaves R in W^T and u_j (zeros above j)
+// in out[0]; out[1]: two columns of workspace.
+template <int LPC, int KR, bool SMALL>
 __device__ __noinline__ void panel_factor(double* W, const int* s_rem, const int* s_sel, int N,
                                           int j0, int m, int nb, int LDU, double* const* out,
                                           double* s_beta, double* s_gam, double* s_uj) {
@@ -314,7 +316,7 @@ __device__ __noinline__ void panel_factor(double* W, const int* s_rem, const int
     x[k] = own && r < m ? col[r] : 0.0;
   }
   for (int j = 0; j < nb; ++j) {
-    double* xj = out[1] + (j & 1) * XS;
+    double* xj = out[1] + (j & 1) * (LPC * KR);
     const bool owner = wid == j / CPW;
     if (owner && pc == j) {                // the column as it is now, zeros above row j
 #pragma unroll
@@ -572,11 +574,14 @@ __global__ void __launch_bounds__(256) qr_init_kernel(const QrTc a) {
 }
 
 // ---- panel ---------------------------------------------------------------------
-// BIG (N > 256): 64 instead of 128 candidates of the pivot search.
+// QP_BIG (N > 256): 64 instead of 128 candidates of the pivot search.  QP_SMALL (N <=
+// 64, many instances): two CTAs an SM (64 registers a thread, 112 KB), as the chain of
+// a step leaves an SM's FP64 pipe idle for two thirds of its 3 to 4 thousand cycles;
+// the same arithmetic.  QP_MID otherwise.
 // PIV: with the pivot search; otherwise the columns in their order (the solver).
-template <bool BIG, bool PIV>
-__global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
-  constexpr int CN = BIG ? 64 : 128;
+template <int SIZE, bool PIV>
+__global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel(const QrTc a, int p) {
+  constexpr int CN = SIZE == QP_BIG ? 64 : 128;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -588,7 +593,7 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
   double* gm = us + NB * LDU;                                  // V^T V
   double* tm = gm + NB * TLD;                                  // T
   double* xs = tm + NB * TLD;                                  // [2][XS]
-  double* s_beta = xs + 2 * XS;
+  double* s_beta = xs + 2 * xs_rows(SIZE == QP_SMALL);
   double* s_gam = s_beta + NB;
   double* s_uj = s_gam + NB;
   float* qf = reinterpret_cast<float*>(s_uj + NB);             // [3][2][row groups][68 or 52]
@@ -607,7 +612,7 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bar + 1);
   int* s_fail = reinterpret_cast<int*>(tmem_holder + 1);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (!DQMC_CHECK(blockDim.x == 512 && N <= (BIG ? QRTC_MAX_N : 256), N) ||
+  if (!DQMC_CHECK(blockDim.x == 512 && N <= (SIZE == QP_BIG ? QRTC_MAX_N : (SIZE == QP_SMALL ? 64 : 256)), N) ||
       !DQMC_CHECK(dyn_smem_bytes() >=
                       (unsigned)(reinterpret_cast<unsigned char*>(s_fail + 1) - smem_raw), m))
     return;
@@ -657,13 +662,16 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
 #define DQMC_SEARCH(TPC_, KM_)                                                                 \
   do {                                                                                         \
     if (Drow)                                                                                  \
-      pivot_search<TPC_, KM_, true>(W, Din, a.lnrm(z), s_rem, s_cand, N, j0, m, nb, qf, s_inv, \
+      pivot_search<TPC_, KM_, true, SIZE == QP_SMALL>(W, Din, a.lnrm(z), s_rem, s_cand, N, j0, m, nb, qf, s_inv, \
                                     s_max, s_sel, s_rho);                                      \
     else                                                                                       \
-      pivot_search<TPC_, KM_, false>(W, Din, a.lnrm(z), s_rem, s_cand, N, j0, m, nb, qf, s_inv, \
+      pivot_search<TPC_, KM_, false, SIZE == QP_SMALL>(W, Din, a.lnrm(z), s_rem, s_cand, N, j0, m, nb, qf, s_inv, \
                                      s_max, s_sel, s_rho);                                     \
   } while (0)
-    if (BIG) {
+    if constexpr (SIZE == QP_SMALL) {
+      if (m <= 32) DQMC_SEARCH(4, 8);
+      else DQMC_SEARCH(4, 16);
+    } else if constexpr (SIZE == QP_BIG) {
       if (m <= 64) DQMC_SEARCH(8, 8);
       else if (m <= 128) DQMC_SEARCH(8, 16);
       else if (m <= 256) DQMC_SEARCH(8, 32);
@@ -699,16 +707,21 @@ __global__ void __launch_bounds__(512, 1) qr_panel_kernel(const QrTc a, int p) {
 #define DQMC_FACTOR(LPC_, KR_)                                                          \
   do {                                                                                  \
     if (wid < LPC_)                                                                     \
-      panel_factor<LPC_, KR_>(W, s_rem, s_sel, N, j0, m, nb, LDU, out, s_beta, s_gam, s_uj); \
+      panel_factor<LPC_, KR_, SIZE == QP_SMALL>(W, s_rem, s_sel, N, j0, m, nb, LDU, out, s_beta, s_gam, s_uj); \
   } while (0)
   {
     double* out[2] = {us, xs};
-    if (m <= 32) DQMC_FACTOR(8, 4);
-    else if (m <= 64) DQMC_FACTOR(8, 8);
-    else if (m <= 128) DQMC_FACTOR(16, 8);
-    else if (m <= 192) DQMC_FACTOR(16, 12);
-    else if (m <= 256) DQMC_FACTOR(16, 16);
-    else DQMC_FACTOR(16, 24);
+    if constexpr (SIZE == QP_SMALL) {
+      if (m <= 32) DQMC_FACTOR(8, 4);
+      else DQMC_FACTOR(8, 8);
+    } else {
+      if (m <= 32) DQMC_FACTOR(8, 4);
+      else if (m <= 64) DQMC_FACTOR(8, 8);
+      else if (m <= 128) DQMC_FACTOR(16, 8);
+      else if (m <= 192) DQMC_FACTOR(16, 12);
+      else if (m <= 256) DQMC_FACTOR(16, 16);
+      else DQMC_FACTOR(16, 24);
+    }
   }
 #undef DQMC_FACTOR
   __syncthreads();
@@ -1179,8 +1192,8 @@ namespace {
 size_t apply_smem(int nkb) {
   return 1024 + RING + 11 * DT + (size_t)32 * (32 * nkb + 1) * 8 + 3 * NB * TLD * 8 + 64 * nkb * 4 + 512;
 }
-size_t panel_smem(int N, int nkb) {
-  return 1024 + RING + ((size_t)NB * (32 * nkb + 1) + 2 * NB * TLD + 2 * XS + 3 * NB) * 8 +
+size_t panel_smem(int N, int nkb, bool small = false) {
+  return 1024 + RING + ((size_t)NB * (32 * nkb + 1) + 2 * NB * TLD + 2 * xs_rows(small) + 3 * NB) * 8 +
          (3 * QF + 2 + 2 * N + 128 + 3 * NB + 64 * nkb + 32) * 4 + 64;
 }
 }  // namespace
@@ -1421,16 +1434,16 @@ cudaError_t solve_tc(const LuArgs& l, void* ws, int slots, cudaStream_t st) {
                          32 * a.nkb * 4 + 512;
   cudaError_t e;
   if ((e = allow_dyn_smem(qr_apply_kernel<APPLY_NEXT>)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_panel_kernel<false, false>)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_panel_kernel<true, false>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<QP_MID, false>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<QP_BIG, false>)) != cudaSuccess) return e;
   if ((e = allow_dyn_smem(solve_back_kernel)) != cudaSuccess) return e;
   if (slots > 65535) slots = 65535;
   for (a.b0 = 0; a.b0 < l.batch; a.b0 += slots) {
     const int nz = l.batch - a.b0 < slots ? l.batch - a.b0 : slots;
     solve_init_kernel<<<dim3((a.nc + 31) / 32, nz), 256, 0, st>>>(a, l);
     for (int p = 0; p < a.np; ++p) {
-      if (N <= 256) qr_panel_kernel<false, false><<<nz, 512, sm_panel, st>>>(a, p);
-      else qr_panel_kernel<true, false><<<nz, 512, sm_panel, st>>>(a, p);
+      if (N <= 256) qr_panel_kernel<QP_MID, false><<<nz, 512, sm_panel, st>>>(a, p);
+      else qr_panel_kernel<QP_BIG, false><<<nz, 512, sm_panel, st>>>(a, p);
       const int left = a.nc - (NB * (p + 1) < N ? NB * (p + 1) : N);
       if (left > 0) qr_apply_kernel<APPLY_NEXT><<<dim3((left + 31) / 32, nz), 512, sm_apply, st>>>(a, p);
     }
@@ -1466,20 +1479,31 @@ cudaError_t qrp_tc(const QrpArgs& q, void* ws, int slots, cudaStream_t st) {
   a.ws = static_cast<unsigned char*>(ws);
   const int LD = 32 * a.nkb + 1;
   const size_t sm_init = (size_t)32 * LD * 8;
-  const size_t sm_apply = apply_smem(a.nkb), sm_panel = panel_smem(N, a.nkb);
+  const size_t sm_apply = apply_smem(a.nkb);
   cudaError_t e;
   if ((e = allow_dyn_smem(qr_init_kernel)) != cudaSuccess) return e;
   if ((e = allow_dyn_smem(qr_apply_kernel<APPLY_REM>)) != cudaSuccess) return e;
   if ((e = allow_dyn_smem(qr_apply_kernel<APPLY_Q>)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_panel_kernel<false, true>)) != cudaSuccess) return e;
-  if ((e = allow_dyn_smem(qr_panel_kernel<true, true>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<QP_SMALL, true>)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(qr_panel_kernel<QP_SMALL, true>,
+                                cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess)
+    return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<QP_MID, true>)) != cudaSuccess) return e;
+  if ((e = allow_dyn_smem(qr_panel_kernel<QP_BIG, true>)) != cudaSuccess) return e;
   if (slots > 65535) slots = 65535;
   for (a.b0 = 0; a.b0 < q.batch; a.b0 += slots) {
     const int nz = q.batch - a.b0 < slots ? q.batch - a.b0 : slots;
+    // Two CTAs an SM where the launch alone covers three quarters of them (another one
+    // runs beside it).  N = 64, M = 100: equal-time chains of 256 instances (128 a launch)
+    // 8.82 -> 8.18 ms, both stacks of the time-displaced call 22.0 -> 20.2 ms; with 96 a
+    // launch 16.1 -> 16.3 ms and with 16, where a CTA's own chain counts, 4.65 -> 4.93.
+    const bool small = N <= 64 && 4 * nz > 3 * device_sms();
+    const size_t sm_panel = panel_smem(N, a.nkb, small);
     qr_init_kernel<<<dim3(a.nkb, nz), 256, sm_init, st>>>(a);
     for (int p = 0; p < a.np; ++p) {
-      if (N <= 256) qr_panel_kernel<false, true><<<nz, 512, sm_panel, st>>>(a, p);
-      else qr_panel_kernel<true, true><<<nz, 512, sm_panel, st>>>(a, p);
+      if (small) qr_panel_kernel<QP_SMALL, true><<<nz, 512, sm_panel, st>>>(a, p);
+      else if (N <= 256) qr_panel_kernel<QP_MID, true><<<nz, 512, sm_panel, st>>>(a, p);
+      else qr_panel_kernel<QP_BIG, true><<<nz, 512, sm_panel, st>>>(a, p);
       const int left = N - NB * (p + 1);
       if (left > 0) qr_apply_kernel<APPLY_REM><<<dim3((left + 31) / 32, nz), 512, sm_apply, st>>>(a, p);
     }
