@@ -52,6 +52,16 @@ def bf16_peak_tflops():
         return 1700.0, "fallback (sustained)"
 
 
+# FP64 products run as 36 exact BF16 digit-pair products on the tensor cores from
+# this N on (below it on the FP64 pipe), in the chain precisions FP64 and BF16x8.
+TENSOR_MIN_N = 33
+DIGIT_PAIRS = 36
+
+
+def products_on_tensor_cores(N: int, prec: int) -> bool:
+    return N >= TENSOR_MIN_N and prec in (0, 8)
+
+
 WORKLOADS = {
     # equal-time G + log det (the headline workload)
     "n256_beta20": dict(L=16, U=4.0, dtau=0.1, beta=20.0, k=10, batch=128, config=4),
@@ -225,15 +235,15 @@ class ClockSampler:
                 "samples": len(self.rows)}
 
 
-def kernel_source_hash(src: str = "gemm_f64.cu") -> str:
+def kernel_source_hash(src: str = "gemm_tc.cu") -> str:
     h = hashlib.sha256()
     with open(os.path.join(ROOT, "paper_2003_05286_gb300", "csrc", src), "rb") as fh:
         h.update(fh.read())
     return h.hexdigest()[:16]
 
 
-def measured_traffic(workload: str, record: str = "chain_gemm_traffic.json",
-                     src: str = "gemm_f64.cu"):
+def measured_traffic(workload: str, record: str = "chain_tc_traffic.json",
+                     src: str = "gemm_tc.cu"):
     """DRAM bytes per launch of the dominant kernel from the committed ncu summary
     (profiles/<record>), or None when the kernel source changed since the capture."""
     path = os.path.join(ROOT, "profiles", record)
@@ -614,7 +624,8 @@ def run_gpu(args, wl, rank, world):
         h.profile_reset()
         step()
         torch.cuda.synchronize()
-        c_ms, c_n, c_fl = h.profile_read(h.PROF_QRP if prec else h.PROF_CHAIN)
+        on_tc = products_on_tensor_cores(N, prec)
+        c_ms, c_n, c_fl = h.profile_read(h.PROF_CHAIN if on_tc or prec == 0 else h.PROF_QRP)
         h.profile(False)
         h.set_graph_mode(graphs)
         if prev is None:
@@ -622,8 +633,9 @@ def run_gpu(args, wl, rank, world):
         else:
             os.environ["DQMC_PIPELINE"] = prev
         if c_ms > 0:
-            u_ach = c_fl / (c_ms / 1e3) / 1e12
-            unshared = {"achieved": u_ach, "frac": u_ach / fp64_peak, "launches": c_n,
+            u_ach = c_fl * (DIGIT_PAIRS if on_tc else 1) / (c_ms / 1e3) / 1e12
+            unshared = {"achieved": u_ach, "launches": c_n,
+                        "frac": u_ach / (bf16_peak_tflops()[0] if on_tc else fp64_peak),
                         "avg_launch_ms": c_ms / max(c_n, 1),
                         "note": "same kernel in one extra step with the sub-batch pipeline off "
                                 "(full batch per launch, no concurrent kernels); not timed"}
@@ -716,32 +728,42 @@ def run_gpu(args, wl, rank, world):
                "api": "dqmc_greens, DQMC_PTR_HOST (pinned host buffers)"}
         he.close()
 
-    if prec == 0:
-        # dominant kernel: the FP64 slice product
+    # dominant kernel: the slice product, except that the pivoted QR dominates a step
+    # whose chain runs on few digits
+    tc = products_on_tensor_cores(N, prec)
+    traffic = None
+    if tc or prec == 0:
         dom_ms, dom_n, dom_flops = chain_ms, chain_n, chain_flops
-        dom_kernel = "gemm_f64_kernel (slice-chain product, 2N^3 x batch flops per launch)"
-        traffic = measured_traffic(args.workload)
+        dom_kernel = "slice-chain product, 2N^3 x batch flops per launch (FP64 pipe)"
+        if tc:
+            dom_kernel = (f"{'chain_tc_kernel' if N <= 128 else 'tc_gemm_kernel'} (slice-chain product: "
+                          f"{DIGIT_PAIRS} exact BF16 digit-pair products of 2N^3 x batch flops)")
+            traffic = measured_traffic(args.workload)
     else:
-        # products on the tensor cores: the FP64 pivoted QR dominates the step
         dom_ms, dom_n, dom_flops = qr_ms, qr_n, qr_flops
-        dom_kernel = "qrp_fused_kernel (pivoted QR incl. forming Q, 8N^3/3 x batch flops per launch)"
-        traffic = measured_traffic(f"{args.workload}_bf16x{prec}", "qrp_fused_traffic.json",
-                                   "qrp_f64.cu")
+        dom_kernel = "pivoted QR incl. forming Q, 8N^3/3 x batch flops per launch"
     achieved = (dom_flops / (dom_ms / 1e3)) / 1e12 if dom_ms > 0 else None
+    dom_peak = fp64_peak
+    if tc:
+        dom_peak = bf16_peak_tflops()[0]
+        achieved = achieved * DIGIT_PAIRS if achieved else None
     roof_tensor = None
     if prec > 0 and chain_ms > 0:
-        pairs = prec * (prec + 1) // 2          # digit pairs p + q <= s + 1
+        pairs = DIGIT_PAIRS if tc else prec * (prec + 1) // 2   # digit pairs p + q <= s + 1
         t_ach = chain_flops * pairs / (chain_ms / 1e3) / 1e12
         t_peak, t_src = bf16_peak_tflops()
         roof_tensor = {"bound": "tensor", "achieved": t_ach, "peak": t_peak, "unit": "TFLOP/s",
                        "frac": t_ach / t_peak, "traffic": None,
-                       "kernel": f"ozaki_gemm_kernel ({pairs} BF16 digit-pair products of 2N^3 per "
+                       "kernel": dom_kernel if tc else
+                                 f"ozaki_gemm_kernel ({pairs} BF16 digit-pair products of 2N^3 per "
                                  "slice product and instance)",
                        "launches": chain_n, "avg_launch_ms": chain_ms / max(chain_n, 1),
                        "peak_source": t_src}
     peak_src = (f"measured: DFMA loop kernel (dqmc_selftest_fp64_rate) on this GPU before the "
                 f"timed region, median SM clock {peak['clocks']['sm_mhz'] if peak['clocks'] else 'n/a'} MHz"
                 f" (derived 152 SM x 4 flop/clk x 2070 MHz = {FP64_DERIVED_TFLOPS:.3f} TFLOP/s)")
+    if tc:
+        peak_src = "dense BF16 GEMM, " + bf16_peak_tflops()[1]
     line = {
         "metric": "greens_functions_per_second", "value": value, "unit": "G/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -753,16 +775,17 @@ def run_gpu(args, wl, rank, world):
                    "l2": "flushed between timed steps (256 MB write)"},
         "fp64_tflops": fl * batch * world * args.steps / (tot_ms / 1e3) / 1e12,
         "fp64_frac_of_peak": fl * batch * args.steps / (tot_ms / 1e3) / 1e12 / fp64_peak,
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": fp64_peak,
-                     "unit": "TFLOP/s", "frac": (achieved / fp64_peak) if achieved else None,
+        "roofline": {"bound": "tensor" if tc else "alu", "achieved": achieved, "peak": dom_peak,
+                     "unit": "TFLOP/s", "frac": (achieved / dom_peak) if achieved else None,
                      "traffic": traffic,
                      "kernel": dom_kernel,
                      "launches": dom_n, "avg_launch_ms": dom_ms / max(dom_n, 1),
                      "stream_time_share": dom_ms / tot_ms if tot_ms > 0 else None,
                      "unshared": unshared,
                      "peak_source": peak_src,
-                     "peak_derived": FP64_DERIVED_TFLOPS,
-                     "frac_of_derived": (achieved / FP64_DERIVED_TFLOPS) if achieved else None},
+                     "peak_derived": None if tc else FP64_DERIVED_TFLOPS,
+                     "frac_of_derived": (achieved / FP64_DERIVED_TFLOPS) if achieved and not tc
+                                        else None},
         "fp64_peaks_measured": peak,
         "roofline_tensor": roof_tensor,
         "gpu_launches": launches_per_step * args.steps,
@@ -889,6 +912,7 @@ def measure_other(args, wl, rank, world, peak=None):
             def step():
                 return dq.greens(K, wl["dtau"], V, k, handle=h)
         extra.update(N=N, M=M, k=k)
+    min_n = min(x.N for x in insts)
     metric, unit = METRICS[name]
     for _ in range(args.warmup):
         out = step()
@@ -909,10 +933,13 @@ def measure_other(args, wl, rank, world, peak=None):
     clk = clocks.stop()
     tot = reduce_max(sum(a.elapsed_time(b) for a, b in ev), dev)
     st = out[-1]
-    # FP64 roofline of the step: with the tensor-core chain, only the flops that
-    # stay on the FP64 pipe (QRs, inversions, wraps) count against its peak
-    fl64 = fl if prec == 0 else fl - fl_tc
+    # roofline of the step: where the products run as digit-pair products on the tensor
+    # cores, all flops against the rate those allow; else, with a chain of few digits,
+    # only the flops that stay in FP64 accuracy (QRs, inversions, wraps)
+    tc = prec in (0, 8) and min_n >= TENSOR_MIN_N
+    fl64 = fl if prec == 0 or tc else fl - fl_tc
     ach = fl64 * args.steps / (tot / 1e3) / 1e12
+    peak_step = bf16_peak_tflops()[0] / DIGIT_PAIRS if tc else fp64_peak
     line = {"metric": metric, "value": job_value(batch, world, args.steps, tot), "unit": unit,
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": tot / args.steps, "higher_is_better": True, "scaling": "weak",
@@ -921,12 +948,14 @@ def measure_other(args, wl, rank, world, peak=None):
             "config": dict(workload=name, baseline_config=wl["config"], instances_per_gpu=batch,
                            chain_precision=prec, cuda_graphs=graphs, fold=args.fold,
                            l2="flushed between timed steps (256 MB write)", **extra),
-            "roofline": {"bound": "alu", "achieved": ach, "peak": fp64_peak,
-                         "unit": "TFLOP/s", "frac": ach / fp64_peak, "traffic": None,
-                         "peak_source": "measured (DFMA loop kernel, dqmc_selftest_fp64_rate)",
-                         "frac_of_derived": ach / FP64_DERIVED_TFLOPS,
+            "roofline": {"bound": "tensor" if tc else "alu", "achieved": ach, "peak": peak_step,
+                         "unit": "TFLOP/s", "frac": ach / peak_step, "traffic": None,
+                         "peak_source": f"dense BF16 GEMM, {bf16_peak_tflops()[1]}, over {DIGIT_PAIRS} "
+                                        "digit-pair products" if tc else
+                                        "measured (DFMA loop kernel, dqmc_selftest_fp64_rate)",
+                         "frac_of_derived": None if tc else ach / FP64_DERIVED_TFLOPS,
                          "kernel": "whole step (all kernels), algorithmic FP64 flops"
-                                   + ("" if prec == 0 else " of the kernels that stay in FP64 (QRs, "
+                                   + ("" if prec == 0 or tc else " of the kernels that stay in FP64 (QRs, "
                                       "inversions, wraps); the chain products and X updates run on "
                                       "the tensor cores and are not counted")},
             "gpu_launches": launches * args.steps, "clocks": clk,
