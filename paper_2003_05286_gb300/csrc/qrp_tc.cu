@@ -46,6 +46,8 @@
 // row r.  V W2 has row exponents (W2 is of order one), and V^T A multiplies
 // 2^{rho_r} u_rj by 2^{-rho_r} a_rc, 2^{rho_r} ~ s_r = Drow_r, so that both
 // factors' largest entries meet in the same row.  Q needs only the first set.
+// T is the first set's in both (the scales go in and out as exponents), so that
+// nothing squares a column's scale: norms over FP64's whole range are taken.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -296,10 +298,16 @@ __device__ __forceinline__ void norm_and_gamma(double sig, double alpha, double&
 // over the sub-partitions; N = 256, 32 columns: 323 -> 240 thousand cycles).  A
 // warp whose columns are done drops out.  Leaves R in W^T and u_j (zeros above j)
 // in out[0]; out[1]: two columns of workspace.
-template <int LPC, int KR, bool SMALL>
-__device__ __noinline__ void panel_factor(double* W, const int* s_rem, const int* s_sel, int N,
+// s_gam[j] is the gamma of u_j 2^{-s_ex[j]}.  Squares of the columns as they are
+// (s_ex = 0) serve while they stay inside FP64's range.  Where one of a panel's steps
+// met one outside (gamma is left at zero) the first form returns true and writes
+// nothing, and WIDE does the panel again from W^T with every pivot column scaled to
+// order one by its largest exponent: one more reduction on the serial chain of a step,
+// which the first form does without.
+template <int LPC, int KR, bool SMALL, bool WIDE>
+__device__ __noinline__ bool panel_factor(double* W, const int* s_rem, const int* s_sel, int N,
                                           int j0, int m, int nb, int LDU, double* const* out,
-                                          double* s_beta, double* s_gam, double* s_uj) {
+                                          double* s_beta, double* s_gam, double* s_uj, int* s_ex) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned FULL = 0xffffffffu;
   constexpr int CPW = 32 / LPC;             // columns per warp
@@ -318,10 +326,22 @@ __device__ __noinline__ void panel_factor(double* W, const int* s_rem, const int
   for (int j = 0; j < nb; ++j) {
     double* xj = out[1] + (j & 1) * (LPC * KR);
     const bool owner = wid == j / CPW;
+    double down = 1.0;                     // the owner's 2^{-ex}, a power of two
+    int mx = 0;
+    if (WIDE && owner) {
+      if (pc == j) {
+#pragma unroll
+        for (int k = 0; k < KR; ++k)
+          if (l8 + LPC * k >= j) mx = max(mx, (int)((__double_as_longlong(x[k]) >> 52) & 0x7ff));
+      }
+      mx = __reduce_max_sync(FULL, mx);
+      down = mx > 0 && mx < 0x7ff ? scalbn(1.0, 1023 - mx) : 1.0;
+      if (lane == 0) s_ex[j] = mx > 0 && mx < 0x7ff ? mx - 1023 : 0;
+    }
     if (owner && pc == j) {                // the column as it is now, zeros above row j
 #pragma unroll
       for (int k = 0; k < KR; ++k)
-        xj[l8 + LPC * k] = l8 + LPC * k >= j ? x[k] : 0.0;
+        xj[l8 + LPC * k] = l8 + LPC * k >= j ? (WIDE ? x[k] * down : x[k]) : 0.0;
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * LPC) : "memory");
     double d = 0.0, ajc = 0.0;
@@ -339,17 +359,20 @@ __device__ __noinline__ void panel_factor(double* W, const int* s_rem, const int
       for (int k = 0; k < 32 / LPC; ++k)     // row j of the column (by row number, as above)
         if (l8 + LPC * k == j) ajc = x[k];
       ajc = __shfl_sync(FULL, ajc, lane / LPC * LPC + j % LPC);
-      if (owner) {                         // the column's own dot is ||x||^2
-        const double sig = __shfl_sync(FULL, d, j % CPW * LPC);
-        const double alpha = __shfl_sync(FULL, ajc, j % CPW * LPC);
+      if (owner) {                         // the column's own dot is ||x||^2 (2^{-ex} of it)
+        const double own_d = __shfl_sync(FULL, d, j % CPW * LPC);
+        const double own_a = __shfl_sync(FULL, ajc, j % CPW * LPC);
+        const double sig = WIDE ? own_d * down : own_d, alpha = WIDE ? own_a * down : own_a;
         double beta = 0.0, gam = 0.0;
-        // a column whose square is out of FP64's range (or zero, or NaN) keeps H = 1
-        if (sig > 1e-290 && sig < 1e300) {
+        if (WIDE ? mx > 0 && mx < 0x7ff : sig > 1e-290 && sig < 1e300) {
           double nrm;
           norm_and_gamma(sig, alpha, nrm, gam);
           beta = alpha >= 0.0 ? -nrm : nrm;
         } else {
-          beta = sig < 1e300 ? alpha : sig;   // a NaN or inf reaches D
+          // nothing to reduce (no normal entry), or a NaN or inf that is to reach D (without
+          // WIDE the panel is done again)
+          if (WIDE) beta = mx == 0 ? alpha : __longlong_as_double(0x7ff8000000000000ll);
+          else beta = sig < 1e300 ? alpha : sig;
         }
         if (lane == 0) { s_beta[j] = beta; s_gam[j] = gam; s_uj[j] = gam > 0.0 ? alpha - beta : 0.0; }
       }
@@ -366,14 +389,18 @@ __device__ __noinline__ void panel_factor(double* W, const int* s_rem, const int
       }
     }
   }
+  // (written before the last barrier of the loop: every warp sees the same)
+  if (!WIDE && __any_sync(FULL, lane < nb && s_gam[lane] == 0.0)) return true;
+  const double up = WIDE && own ? scalbn(1.0, s_ex[pc]) : 1.0;
 #pragma unroll
   for (int k = 0; k < KR; ++k) {
     const int r = l8 + LPC * k;
     if (r < rows) {
-      us[r] = own && r < m && r >= pc && s_gam[pc] > 0.0 ? (r == pc ? s_uj[pc] : x[k]) : 0.0;
-      if (own && r <= pc && r < m) col[r] = r == pc ? s_beta[pc] : x[k];
+      us[r] = own && r < m && r >= pc && s_gam[pc] > 0.0 ? (r == pc ? (WIDE ? s_uj[pc] * up : s_uj[pc]) : x[k]) : 0.0;
+      if (own && r <= pc && r < m) col[r] = r == pc ? (WIDE ? s_beta[pc] * up : s_beta[pc]) : x[k];
     }
   }
+  return false;
 }
 
 // Waits on a phase unless an earlier wait of this CTA already gave up.
@@ -492,7 +519,8 @@ struct QrTc {
   __host__ __device__ double* T(int z, int p, int set) const {
     return reinterpret_cast<double*>(v(z, np, set)) + p * (NB * NB);
   }
-  // exponents of the second set: f_j of V^T's rows, e_r of V's rows
+  // exponents: f_j of V^T's rows (in the first set the scales of its vectors), in the
+  // second set also e_r of V's rows
   __host__ __device__ int* f(int z, int p, int set) const {
     return reinterpret_cast<int*>(T(z, np, set)) + p * NB;
   }
@@ -602,7 +630,9 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   int* s_rem = reinterpret_cast<int*>(s_key + N);              // [m]
   int* s_cand = s_rem + N;                                     // [CN] positions in rem
   int* s_sel = s_cand + CN;                                    // [32] candidate numbers
-  int* s_f = s_sel + NB;                                       // [32] exponents of V^T's rows
+  int* s_ex = s_sel + NB;                                      // [32] exponents of gamma's vectors
+  int* s_f0 = s_ex + NB;                                       // [32] the first set's s_f
+  int* s_f = s_f0 + NB;                                        // [32] exponents of V^T's rows
   int* s_h = s_f + NB;                                         // [32] of V's columns times 2^{-rho_r}
   int* s_rho = s_h + NB;                                       // [32 nkl]
   int* s_er = s_rho + 32 * nkl;                                // [32 nkl] exponents of V's rows
@@ -635,6 +665,7 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   // ---- candidates: the CN remaining columns of largest key (ties: lowest place)
   const double* Drow = a.q.Drow ? a.q.Drow + (long long)b * a.q.sDrow : nullptr;
   if (tid < 32 * nkl) s_rho[tid] = row_rho(Drow, j0 + tid, N);
+  if (tid < NB) s_ex[tid] = 0;
   if (!PIV && tid < NB) {
     s_rem[tid] = j0 + tid;
     s_sel[tid] = tid;
@@ -704,10 +735,17 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   }
   // ---- FP64 Householder panel (rows per lane rounded up: straight-line loops, as a
   // predicated FP64 instruction holds the pipe like any other) ---------------------
-#define DQMC_FACTOR(LPC_, KR_)                                                          \
-  do {                                                                                  \
-    if (wid < LPC_)                                                                     \
-      panel_factor<LPC_, KR_, SIZE == QP_SMALL>(W, s_rem, s_sel, N, j0, m, nb, LDU, out, s_beta, s_gam, s_uj); \
+#define DQMC_FACTOR(LPC_, KR_)                                                                    \
+  do {                                                                                            \
+    bool redo = false;                                                                            \
+    if (wid < LPC_)                                                                               \
+      redo = panel_factor<LPC_, KR_, SIZE == QP_SMALL, false>(W, s_rem, s_sel, N, j0, m, nb, LDU, \
+                                                              out, s_beta, s_gam, s_uj, s_ex);    \
+    if (redo) {                             /* (alike in these warps) */                          \
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * LPC_) : "memory");                                \
+      panel_factor<LPC_, KR_, SIZE == QP_SMALL, true>(W, s_rem, s_sel, N, j0, m, nb, LDU, out,    \
+                                                      s_beta, s_gam, s_uj, s_ex);                 \
+    }                                                                                             \
   } while (0)
   {
     double* out[2] = {us, xs};
@@ -760,7 +798,8 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
       if (l == 0) {
         s_f[c] = bad ? TC_NONFINITE : (mf == 0 ? 0 : mf - 100000 - 1020);
         s_h[c] = bad ? TC_NONFINITE : (mf == 0 ? 0 : mh - 1020);
-        if (set) a.f(z, p, 1)[c] = s_f[c];
+        if (!set) s_f0[c] = s_f[c];
+        a.f(z, p, set)[c] = s_f[c];
       }
     }
     __syncthreads();
@@ -820,15 +859,15 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
       for (int c0 = 16 * (wid >> 2); c0 < 16 * (wid >> 2) + 16; c0 += 8) stacked_partial(tmem, wid, c0, ex);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    // V^T V; in the first set of the scaled vectors (exponent 0), whose gamma is
-    // gamma_j 2^{2 f_j}
+    // V^T V of the vectors the first set holds, u_j 2^{-f_j} (in that set exponent 0), in
+    // the second one too: entries and T's stay of order one whatever the columns' scales
     for (int e = tid; e < NB * NB; e += 512) {
       const int i = e & 31, c = e >> 5;
-      gm[i * TLD + c] = stacked_value(ex, i, c, set ? s_h[i] + s_f[c] : 0);
+      gm[i * TLD + c] = stacked_value(ex, i, c, set ? s_h[i] + s_f[c] - s_f0[i] - s_f0[c] : 0);
     }
-    double* s_g = xs;                       // (xs is free)
-    if (tid < NB)
-      s_g[tid] = tid < nb && s_f[tid] < TC_NONFINITE / 2 ? (set ? s_gam[tid] : scalbn(s_gam[tid], 2 * s_f[tid])) : 0.0;
+    double* s_g = xs;                       // (xs is free) gamma_j 2^{2 f_j}
+    if (!set && tid < NB)
+      s_g[tid] = tid < nb && s_f[tid] < TC_NONFINITE / 2 ? scalbn(s_gam[tid], 2 * (s_f[tid] - s_ex[tid])) : 0.0;
     for (int e = tid; e < NB * TLD; e += 512) tm[e] = 0.0;
     __syncthreads();
     // ---- T: T_jj = gamma_j, T(:j, j) = -gamma_j T(:j,:j) G(:j, j); 8 x 8 blocks by one
@@ -906,7 +945,9 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
   int* ecol = reinterpret_cast<int*>(tt + NB * TLD);            // [32]
   int* ew = ecol + 32;
   int* s_f = ew + 32;                                           // [32]
-  int* s_rho = s_f + 32;                                        // [32 nkb]
+  int* s_f0 = s_f + 32;                                         // [32]
+  double* s_dn = reinterpret_cast<double*>(s_f0 + 32);          // [32] 2^{-f0}
+  int* s_rho = reinterpret_cast<int*>(s_dn + 32);               // [32 nkb]
   int* s_er = s_rho + 32 * a.nkb;                               // [32 nkb]
   uint64_t* full = reinterpret_cast<uint64_t*>(s_er + 32 * a.nkb);
   uint64_t* done = full + 1;
@@ -972,6 +1013,8 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
     if (tid < 32) {
       ew[tid] = 0;
       s_f[tid] = set ? a.f(z, pp, 1)[tid] : 0;
+      s_f0[tid] = set ? a.f(z, pp, 0)[tid] : 0;
+      s_dn[tid] = set ? scalbn(1.0, -s_f0[tid]) : 1.0;
     }
     for (int r = tid; r < 32 * a.nkb; r += 512) {
       s_rho[r] = set ? row_rho(Drow, r, N) : 0;
@@ -1033,7 +1076,7 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
     for (int e = tid; e < NB * NB; e += 512) {
       const int i = e & 31, c = e >> 5, ec = ecol[c] + s_f[i];
       w1[i * TLD + c] = ec >= TC_NONFINITE / 2 ? __longlong_as_double(0x7ff8000000000000ll)
-                                           : stacked_value(ex, i, c, ec);
+                                           : stacked_value(ex, i, c, ec - s_f0[i]);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -1065,7 +1108,8 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
           }
           if (l <= i) s0 = fma(tt[l * TLD + i], w1[l * TLD + lane], s0);
         }
-        const double s = s0 + s1;
+        double s = s0 + s1;
+        if (set) s *= s_dn[i];               // V's digits are those of u itself
         w2[i * TLD + lane] = s;
         atomicMax(&ew[lane], (int)((__double_as_longlong(s) >> 52) & 0x7ff));
       }
@@ -1190,11 +1234,11 @@ __global__ void __launch_bounds__(256) qr_out_kernel(const QrTc a) {
 
 namespace {
 size_t apply_smem(int nkb) {
-  return 1024 + RING + 11 * DT + (size_t)32 * (32 * nkb + 1) * 8 + 3 * NB * TLD * 8 + 64 * nkb * 4 + 512;
+  return 1024 + RING + 11 * DT + (size_t)32 * (32 * nkb + 1) * 8 + 3 * NB * TLD * 8 + 64 * nkb * 4 + 896;
 }
 size_t panel_smem(int N, int nkb, bool small = false) {
   return 1024 + RING + ((size_t)NB * (32 * nkb + 1) + 2 * NB * TLD + 2 * xs_rows(small) + 3 * NB) * 8 +
-         (3 * QF + 2 + 2 * N + 128 + 3 * NB + 64 * nkb + 32) * 4 + 64;
+         (3 * QF + 2 + 2 * N + 128 + 5 * NB + 64 * nkb + 32) * 4 + 64;
 }
 }  // namespace
 
