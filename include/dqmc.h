@@ -140,6 +140,8 @@ dqmc_status dqmc_set_gemm_tile(dqmc_handle h, int tile);
  *                         the device's SM count (152 on GB300) and
  *                         ceil(M/k) >= 4, else sequential.
  * Both give G and log det of the same definition; they differ by rounding.
+ * With BF16X8 a call whose tree does not fit (device memory, memory limit) is
+ * folded sequentially; with FP64 it returns DQMC_ERR_NOMEM.
  * Invalid mode: DQMC_ERR_ARG. */
 typedef enum { DQMC_FOLD_SEQUENTIAL = 0, DQMC_FOLD_TREE = 1, DQMC_FOLD_AUTO = 2 } dqmc_fold_mode;
 dqmc_status dqmc_set_chain_fold(dqmc_handle h, int mode);

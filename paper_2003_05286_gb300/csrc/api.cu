@@ -86,9 +86,9 @@ struct dqmc_handle_s {
   // cap on the device bytes all of the above may hold together (0: none);
   // growth past it fails with DQMC_ERR_NOMEM before any buffer is released
   size_t mem_limit = 0;
-  // set while a call that found no room for the digits of tensor-core FP64
-  // products runs without them
-  bool no_tc = false;
+  // what a call that found no room is recorded without (see place): 0 nothing, 1 the
+  // scratch of the tensor-core kernels, 2 (BF16X8) also the tree fold
+  int lean = 0;
 };
 
 namespace {
@@ -150,21 +150,24 @@ dqmc_status ensure_ws(dqmc_handle h, size_t bytes) {
   return DQMC_OK;
 }
 
-// Sizes the workspace by layout(arena) and lays it out.  tc (whether the layout
-// holds digits of tensor-core products) is dropped when there is no room for
-// them: the call then runs those products on the FP64 pipe.
+// The last step of the ladder: BF16X8 may be folded either way (its chain precision
+// alone used to mean the sequential fold, whose workspace is the smaller one); an FP64
+// call whose tree fold does not fit is refused.
+inline int max_lean(dqmc_handle h) { return h->prec == DQMC_CHAIN_BF16X8 ? 2 : 1; }
+
+// Sizes the workspace by layout(arena) and lays it out.  Where there is no room, lean
+// goes up and the layout, which reads it, is asked again: from 1 on it holds no digits
+// for tensor-core kernels (their work runs on the FP64 pipe), at 2 no tree fold.
 template <class F>
-dqmc_status place(dqmc_handle h, bool& tc, F&& layout) {
-  Arena measure;
-  layout(measure);
-  dqmc_status rc = ensure_ws(h, measure.off);
-  if (rc == DQMC_ERR_NOMEM && tc && !h->capturing) {
-    tc = false;
-    Arena again;
-    layout(again);
-    rc = ensure_ws(h, again.off);
+dqmc_status place(dqmc_handle h, int& lean, F&& layout) {
+  while (true) {
+    Arena measure;
+    layout(measure);
+    const dqmc_status rc = ensure_ws(h, measure.off);
+    if (rc == DQMC_OK) break;
+    if (rc != DQMC_ERR_NOMEM || h->capturing || lean >= max_lean(h)) return rc;
+    ++lean;
   }
-  if (rc != DQMC_OK) return rc;
   Arena ar;
   ar.base = h->ws;
   layout(ar);
@@ -391,7 +394,7 @@ constexpr long long TC_SCRATCH = 512LL << 20;   // bytes of digits a TcWs may ho
 constexpr int TC_SHARES = 8;                    // products side by side (kMaxJobs)
 
 inline bool tc_wanted(dqmc_handle h, int N) {
-  return !h->no_tc && N >= TC_MIN_N && N <= TC_MAX_N;
+  return h->lean < 1 && N >= TC_MIN_N && N <= TC_MAX_N;
 }
 
 // Digits of the reduced-precision chain (ozaki_tc.cu), 0 for products in FP64
@@ -402,11 +405,11 @@ inline bool tc_wanted(dqmc_handle h, int N) {
 // 2^-51 of row max x column max.  Equal-time chain, M = 100, k = 5: N = 9, 64
 // instances 4.69 -> 0.99 ms, N = 25, 256 instances 8.94 -> 4.43, N = 36, 256
 // instances 12.6 -> 9.4; one instance (tree fold) N = 256 39.9 -> 15.7.  Only a
-// call that had no room for the tensor cores' scratch under capture (no_tc) still
+// call that had no room for the tensor cores' scratch under capture (lean) still
 // takes the base-128 digits.
 inline int reduced_digits(dqmc_handle h, int N) {
   if (h->prec == DQMC_CHAIN_FP64) return 0;
-  return h->prec == DQMC_CHAIN_BF16X8 && (!h->no_tc || N < CHAIN_TC_MIN_N) ? 0 : (int)h->prec;
+  return h->prec == DQMC_CHAIN_BF16X8 && (h->lean < 1 || N < CHAIN_TC_MIN_N) ? 0 : (int)h->prec;
 }
 
 // Chunks of the FP64 chain in one tensor-core launch (chain_tc.cu): from N = 33,
@@ -414,7 +417,7 @@ inline int reduced_digits(dqmc_handle h, int N) {
 // k = 10: N = 36 1 instance 1.78 -> 1.75 ms, 32 4.09 -> 3.62, 256 9.07 -> 6.06 ms;
 // N = 49 256 instances 16.3 -> 8.7 ms; N = 100 256 instances 25.2 -> 23.3.
 inline bool chain_tc_wanted(dqmc_handle h, int N) {
-  return !h->no_tc && N >= CHAIN_TC_MIN_N && N <= 128;
+  return h->lean < 1 && N >= CHAIN_TC_MIN_N && N <= 128;
 }
 
 // The shared operand (the slice matrix), all that the fused chain needs.
@@ -550,7 +553,7 @@ struct QrWs {
 };
 
 inline bool qrtc_wanted(dqmc_handle h, int N) {
-  return !h->no_tc && h->decomp == DQMC_DECOMP_QR && N >= QRTC_MIN_N && N <= QRTC_MAX_N;
+  return h->lean < 1 && h->decomp == DQMC_DECOMP_QR && N >= QRTC_MIN_N && N <= QRTC_MAX_N;
 }
 
 void take_qr(Arena& ar, long long batch, int N, int row_graded, QrWs& w) {
@@ -1530,12 +1533,12 @@ static dqmc_status graph_call(dqmc_handle h, GraphKey key, F&& body) {
   if (!h->gstream && cudaStreamCreateWithFlags(&h->gstream, cudaStreamNonBlocking) != cudaSuccess)
     return DQMC_ERR_CUDA;
   cudaStream_t caller = h->stream;
-  h->no_tc = false;
-  struct Restore {   // no_tc holds for this call only
+  h->lean = 0;
+  struct Restore {   // lean holds for this call only
     dqmc_handle h;
-    ~Restore() { h->no_tc = false; }
+    ~Restore() { h->lean = 0; }
   } restore{h};
-  for (int attempt = 0; attempt < 3; ++attempt) {
+  for (int attempt = 0; attempt < 4; ++attempt) {   // as it is, two leaner layouts, grown
     h->stream = h->gstream;
     if (cudaStreamBeginCapture(h->gstream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
       h->stream = caller;
@@ -1554,8 +1557,8 @@ static dqmc_status graph_call(dqmc_handle h, GraphKey key, F&& body) {
       cudaGetLastError();
       const dqmc_status grown = ensure_ws(h, h->ws_need);
       if (grown != DQMC_OK) {
-        if (grown != DQMC_ERR_NOMEM || h->no_tc) return grown;
-        h->no_tc = true;   // record again without the digits of tensor-core products
+        if (grown != DQMC_ERR_NOMEM || h->lean >= max_lean(h)) return grown;
+        ++h->lean;   // record again with less
         continue;
       }
       key.v[key.n - 2] = (unsigned long long)(uintptr_t)h->ws;
@@ -1609,20 +1612,22 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   const bool host = h->pmode == DQMC_PTR_HOST;
   const long long NN = (long long)N * N;
   const int nc = n_chunks(M, k);
-  const bool tree = use_tree(h, batch, N, nc);
-  // padded slice stride of exp(V): one spare chunk, and for the tree every
-  // padding chunk of its power-of-two width
-  const int mp_chunks = tree && tree_width(nc) > nc + 1 ? tree_width(nc) : nc + 1;
-  const long long Mp = (long long)mp_chunks * k;
+  const int digits = reduced_digits(h, N);
+  int lean = h->lean;
+  bool tree = false;
+  long long Mp = 0;
   TreeWs tw;
   PlainWs pw;
-  const int digits = reduced_digits(h, N);
-  const bool tc_gemms = digits == 0 && (!tree || N >= TC_TREE_MIN_N);
-  bool tc = !h->no_tc;
 
   auto layout = [&](Arena& ar, ExpmWs& ew, ChainWs& cw, LohWs& lw, double*& E, double*& expV,
                     double*& U, double*& D, double*& X0, double*& X1, int*& st, HostIO& io,
                     double*& Gd, double*& ldd, int*& sgd) {
+    tree = lean < 2 && use_tree(h, batch, N, nc);
+    const bool tc = lean < 1, tc_gemms = digits == 0 && (!tree || N >= TC_TREE_MIN_N);
+    // padded slice stride of exp(V): one spare chunk, and for the tree every
+    // padding chunk of its power-of-two width
+    const int mp_chunks = tree && tree_width(nc) > nc + 1 ? tree_width(nc) : nc + 1;
+    Mp = (long long)mp_chunks * k;
     take_expm(ar, N, ew);
     E = ew.t0;
     expV = ar.take<double>(Mp * N * batch);
@@ -1661,7 +1666,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   ExpmWs ew; ChainWs cw; LohWs lw; HostIO io;
   double *E, *expV, *U, *D, *X0, *X1, *Gd = nullptr, *ldd = nullptr;
   int *stat, *sgd = nullptr;
-  CKS(place(h, tc, [&](Arena& ar) {
+  CKS(place(h, lean, [&](Arena& ar) {
     layout(ar, ew, cw, lw, E, expV, U, D, X0, X1, stat, io, Gd, ldd, sgd);
   }));
   cudaStream_t st = h->cur;
@@ -2213,8 +2218,9 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
   double *gq[3] = {nullptr, nullptr, nullptr}, *gtmp = nullptr;   // grid values (all_tau)
   int* stat;
   int* shiftd = nullptr;
-  bool tc = !h->no_tc;
+  int lean = h->lean;
   auto layout = [&](Arena& ar) {
+    const bool tc = lean < 1;
     take_expm(ar, N, ew);
     expV = ar.take<double>(Mp * N * batch);
     if (all_tau) {
@@ -2258,7 +2264,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       G0td = G0t ? ar.take<double>(batch * outlen) : nullptr;
     }
   };
-  CKS(place(h, tc, layout));
+  CKS(place(h, lean, layout));
   cudaStream_t st = h->cur;
   const double* Kd = K;
   const double* Vd = V;
@@ -2389,8 +2395,9 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
   ExpmWs ew, ewi; ChainWs cw, cw2; StackWs sw; MidWs mw; LohWs lw; HostIO io;
   double *expV, *expmV, *Gw, *W1, *dVd = nullptr, *ldd = nullptr;
   int *stat, *sgd = nullptr;
-  bool tc = !h->no_tc;
+  int lean = h->lean;
   auto layout = [&](Arena& ar) {
+    const bool tc = lean < 1;
     take_expm(ar, N, ew);
     take_expm(ar, N, ewi);
     expV = ar.take<double>(Mp * N * batch);
@@ -2429,7 +2436,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       sgd = ar.take<int>(batch);
     }
   };
-  CKS(place(h, tc, layout));
+  CKS(place(h, lean, layout));
   cudaStream_t st = h->cur;
   const double* Kd = K;
   const double* Vd = V;
@@ -2577,8 +2584,9 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
   }
   // ---- workspace (h->ws) and index tables (h->rtab): one region per group ----
   std::vector<RaggedGroupWs> gw(groups.size());
-  bool tc = true;
+  int lean = 0;
   auto layout = [&](Arena& ar) {
+    const bool tc = lean < 1;
     for (size_t i = 0; i < groups.size(); ++i) {
       const RaggedGroup& g = groups[i];
       RaggedGroupWs& w = gw[i];
@@ -2618,7 +2626,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
   };
   Arena measure_t;
   layout_tables(measure_t);
-  CKS(place(h, tc, layout));
+  CKS(place(h, lean, layout));
   if (measure_t.off > h->rtab_bytes) {
     if (h->capturing) return DQMC_ERR_UNSUPPORTED;
     if (!within_limit(h, h->rtab_bytes, measure_t.off)) return DQMC_ERR_NOMEM;
