@@ -400,16 +400,14 @@ inline bool tc_wanted(dqmc_handle h, int N) {
 // Digits of the reduced-precision chain (ozaki_tc.cu), 0 for products in FP64
 // accuracy.  Eight BF16 digits per operand are what the FP64 products take too,
 // with 8 instead of 7 bits each, and below N = 33 the FP64 pipe needs less time
-// than any digits: DQMC_CHAIN_BF16X8 runs on the FP64 chain.  One product of 128
-// instances, N = 256: 218 -> 170 us, its split 79 -> 43, error 2^-58 instead of
-// 2^-51 of row max x column max.  Equal-time chain, M = 100, k = 5: N = 9, 64
-// instances 4.69 -> 0.99 ms, N = 25, 256 instances 8.94 -> 4.43, N = 36, 256
-// instances 12.6 -> 9.4; one instance (tree fold) N = 256 39.9 -> 15.7.  Only a
-// call that had no room for the tensor cores' scratch under capture (lean) still
-// takes the base-128 digits.
-inline int reduced_digits(dqmc_handle h, int N) {
-  if (h->prec == DQMC_CHAIN_FP64) return 0;
-  return h->prec == DQMC_CHAIN_BF16X8 && (h->lean < 1 || N < CHAIN_TC_MIN_N) ? 0 : (int)h->prec;
+// than any digits: DQMC_CHAIN_BF16X8 runs on the FP64 chain, also where that has
+// to go without its digits (eager or captured: the same kernels at the same limit).
+// One product of 128 instances, N = 256: 218 -> 170 us, its split 79 -> 43, error
+// 2^-57 instead of 2^-51 of row max x column max.  Equal-time chain, M = 100, k = 5:
+// N = 9, 64 instances 4.69 -> 0.99 ms, N = 25, 256 instances 8.94 -> 4.43, N = 36, 256
+// instances 12.6 -> 9.4; one instance (tree fold) N = 256 39.9 -> 15.7.
+inline int reduced_digits(dqmc_handle h) {
+  return h->prec == DQMC_CHAIN_FP64 || h->prec == DQMC_CHAIN_BF16X8 ? 0 : (int)h->prec;
 }
 
 // Chunks of the FP64 chain in one tensor-core launch (chain_tc.cu): from N = 33,
@@ -1131,8 +1129,8 @@ dqmc_status run_chain_tree(dqmc_handle h, int batch, int N, int M, int k, const 
 // Tree fold for the equal-time chain: by setting, or (auto) when the level-0
 // QRs of all chunks of the batch fit in one wave of CTAs (one per SM) and the
 // chain has at least four chunks.
-bool use_tree(dqmc_handle h, int batch, int N, int nc) {
-  if (reduced_digits(h, N) != 0 || h->decomp != DQMC_DECOMP_QR) return false;
+bool use_tree(dqmc_handle h, int batch, int nc) {
+  if (reduced_digits(h) != 0 || h->decomp != DQMC_DECOMP_QR) return false;
   if (h->fold == DQMC_FOLD_TREE) return nc > 1;
   if (h->fold == DQMC_FOLD_SEQUENTIAL) return false;
   return nc >= 4 && (long long)batch * nc <= h->sms;
@@ -1612,7 +1610,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   const bool host = h->pmode == DQMC_PTR_HOST;
   const long long NN = (long long)N * N;
   const int nc = n_chunks(M, k);
-  const int digits = reduced_digits(h, N);
+  const int digits = reduced_digits(h);
   int lean = h->lean;
   bool tree = false;
   long long Mp = 0;
@@ -1622,7 +1620,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
   auto layout = [&](Arena& ar, ExpmWs& ew, ChainWs& cw, LohWs& lw, double*& E, double*& expV,
                     double*& U, double*& D, double*& X0, double*& X1, int*& st, HostIO& io,
                     double*& Gd, double*& ldd, int*& sgd) {
-    tree = lean < 2 && use_tree(h, batch, N, nc);
+    tree = lean < 2 && use_tree(h, batch, nc);
     const bool tc = lean < 1, tc_gemms = digits == 0 && (!tree || N >= TC_TREE_MIN_N);
     // padded slice stride of exp(V): one spare chunk, and for the tree every
     // padding chunk of its power-of-two width
@@ -2239,7 +2237,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       // the first also serves the products over all stack slots after the chains
       take_tc(ar, Q, N, cw.tc);
       take_tc(ar, batch, N, cw2.tc);
-    } else if (tc && !reduced_digits(h, N) && chain_tc_wanted(h, N)) {
+    } else if (tc && !reduced_digits(h) && chain_tc_wanted(h, N)) {
       take_tc_shared(ar, N, cw.tc);
       take_tc_shared(ar, N, cw2.tc);
     }
@@ -2247,7 +2245,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       take_qr(ar, Q, N, 0, cw.qr);
       take_qr(ar, batch, N, 0, cw2.qr);
     }
-    if (const int digits = reduced_digits(h, N)) {
+    if (const int digits = reduced_digits(h)) {
       take_ozaki(ar, batch, N, digits, cw);
       take_ozaki(ar, batch, N, digits, cw2);
     }
@@ -2410,7 +2408,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       // the first also serves the products over all stack slots after the chains
       take_tc(ar, Q, N, cw.tc);
       take_tc(ar, batch, N, cw2.tc);
-    } else if (tc && !reduced_digits(h, N) && chain_tc_wanted(h, N)) {
+    } else if (tc && !reduced_digits(h) && chain_tc_wanted(h, N)) {
       take_tc_shared(ar, N, cw.tc);
       take_tc_shared(ar, N, cw2.tc);
     }
@@ -2418,7 +2416,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       take_qr(ar, Q, N, 0, cw.qr);
       take_qr(ar, batch, N, 0, cw2.qr);
     }
-    if (const int digits = reduced_digits(h, N)) {
+    if (const int digits = reduced_digits(h)) {
       take_ozaki(ar, batch, N, digits, cw);
       take_ozaki(ar, batch, N, digits, cw2);
     }
@@ -2602,7 +2600,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       take_chain(ar, nb, N, w.cw);
       w.cw.tc = TcWs{};
       w.cw.qr = QrWs{};
-      const int digits = reduced_digits(h, N);
+      const int digits = reduced_digits(h);
       if (tc && !digits && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
       else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, w.cw.tc);
       if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr);

@@ -552,8 +552,7 @@ cudaError_t ozaki_split(const double* X, long long ldm, long long ldj, long long
     case 4: return go(ozaki_split_kernel<4>);
     case 5: return go(ozaki_split_kernel<5>);
     case 6: return go(ozaki_split_kernel<6>);
-    case 7: return go(ozaki_split_kernel<7>);
-    default: return go(ozaki_split_kernel<8>);
+    default: return go(ozaki_split_kernel<7>);
   }
 }
 
@@ -570,7 +569,7 @@ static cudaError_t ozaki_gemm_impl(const __nv_bfloat16* As, const int* eA, long 
                                    const double* csrc = nullptr, long long scsrc = 0) {
   if (sA != 0 && sA < (long long)s * P128 * PK) return cudaErrorInvalidValue;
   if (P128 % OZ_BM || PN % OZ_BN || PK % OZ_BK || PK < OZ_BK) return cudaErrorInvalidValue;
-  if (s < 1 || s > 8) return cudaErrorInvalidValue;
+  if (s < 1 || s > 7) return cudaErrorInvalidValue;
   OzPairs pr = oz_pairs(s, N);
   if (pr.ngroups > 8 || pr.n > 40) return cudaErrorNotSupported;
   // the kernel issues the pairs of one A digit as one wide MMA: it needs one
