@@ -14,6 +14,7 @@
 //   a9-a10  G(tau,tau) and G(tau,0) from the two stacks through one D+/D- split
 //       middle matrix (Eq. (inversion_tdgf_loh)).
 //   a11 gradient 1 - G_l(i,i): checkpoints from the stacks, wrapping in between.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <utility>
@@ -554,13 +555,20 @@ inline bool qrtc_wanted(dqmc_handle h, int N) {
   return h->lean < 1 && h->decomp == DQMC_DECOMP_QR && N >= QRTC_MIN_N && N <= QRTC_MAX_N;
 }
 
-void take_qr(Arena& ar, long long batch, int N, int row_graded, QrWs& w) {
+// Slots for `batch` factorisations, and as many bytes as `solves` solves in one pass
+// take (a solver's slot holds R's digits too: N = 256 3.2 instead of 2.2 MB).
+void take_qr(Arena& ar, long long batch, int N, int row_graded, QrWs& w, long long solves) {
   const long long slot = (long long)qrp_tc_slot_bytes(N, row_graded);
   long long n = TC_SCRATCH / slot;
   batch += TC_SHARES - 1;
   n = batch < n ? batch : (n < TC_SHARES ? TC_SHARES : n);
-  w.bytes = (size_t)(n * slot);
-  w.ws = ar.take<char>(n * slot);
+  long long bytes = n * slot;
+  if (N >= SOLVETC_MIN_N) {
+    const long long s = (long long)solve_tc_slot_bytes(N), m = TC_SCRATCH / s;
+    bytes = std::max(bytes, s * (solves < m ? solves : (m < 1 ? 1 : m)));
+  }
+  w.bytes = (size_t)bytes;
+  w.ws = ar.take<char>(bytes);
 }
 
 QrWs qr_part(const QrWs& w, int q, int nj, int N) {
@@ -1635,7 +1643,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       tw.qr = QrWs{};
       if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, (long long)batch * tw.P0, N, tw.tc);
       else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, tw.tc);
-      if (tc && qrtc_wanted(h, N)) take_qr(ar, (long long)batch * tw.P0, N, 1, tw.qr);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, (long long)batch * tw.P0, N, 1, tw.qr, batch);
       U = D = X0 = X1 = nullptr;
     } else {
       U = ar.take<double>(NN * batch);
@@ -1647,7 +1655,7 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       cw.qr = QrWs{};
       if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, batch, N, cw.tc);
       else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, cw.tc);
-      if (tc && qrtc_wanted(h, N)) take_qr(ar, batch, N, 0, cw.qr);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, batch, N, 0, cw.qr, batch);
     }
     if (digits) take_ozaki(ar, batch, N, digits, cw);
     take_loh(ar, batch, N, lw);
@@ -2242,8 +2250,8 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       take_tc_shared(ar, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
-      take_qr(ar, Q, N, 0, cw.qr);
-      take_qr(ar, batch, N, 0, cw2.qr);
+      take_qr(ar, Q, N, 0, cw.qr, Q);
+      take_qr(ar, batch, N, 0, cw2.qr, 0);
     }
     if (const int digits = reduced_digits(h)) {
       take_ozaki(ar, batch, N, digits, cw);
@@ -2413,8 +2421,8 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       take_tc_shared(ar, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
-      take_qr(ar, Q, N, 0, cw.qr);
-      take_qr(ar, batch, N, 0, cw2.qr);
+      take_qr(ar, Q, N, 0, cw.qr, Q);
+      take_qr(ar, batch, N, 0, cw2.qr, 0);
     }
     if (const int digits = reduced_digits(h)) {
       take_ozaki(ar, batch, N, digits, cw);
@@ -2603,7 +2611,7 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       const int digits = reduced_digits(h);
       if (tc && !digits && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
       else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, w.cw.tc);
-      if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr, nb);
       if (digits) take_ozaki(ar, nb, N, digits, w.cw);
       take_loh(ar, nb, N, w.lw);
       if (h->inv == DQMC_INV_PLAIN) take_plain(ar, nb, N, w.pw);

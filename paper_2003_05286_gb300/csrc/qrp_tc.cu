@@ -1482,6 +1482,8 @@ cudaError_t solve_tc(const LuArgs& l, void* ws, int slots, cudaStream_t st) {
   if ((e = allow_dyn_smem(qr_panel_kernel<QP_BIG, false>)) != cudaSuccess) return e;
   if ((e = allow_dyn_smem(solve_back_kernel)) != cudaSuccess) return e;
   if (slots > 65535) slots = 65535;
+  const int passes = (l.batch + slots - 1) / slots;
+  slots = (l.batch + passes - 1) / passes;   // passes of equal size
   for (a.b0 = 0; a.b0 < l.batch; a.b0 += slots) {
     const int nz = l.batch - a.b0 < slots ? l.batch - a.b0 : slots;
     solve_init_kernel<<<dim3((a.nc + 31) / 32, nz), 256, 0, st>>>(a, l);

@@ -1,0 +1,60 @@
+"""Scratch of the tensor-core kernels: what a call's instances need and no more."""
+import numpy as np
+import pytest
+
+import dqmc_inputs as di
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dq():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2003_05286_gb300 as m
+    m.lib()
+    return m
+
+
+def _dev(x):
+    return torch.tensor(np.ascontiguousarray(x), dtype=torch.float64, device="cuda")
+
+
+def _fields(seed, batch, M, N):
+    return _dev(np.stack([0.3 * di.ising_field(seed + b, M, N) for b in range(batch)]))
+
+
+def _kernels(fn):
+    """Launches of every kernel of one call, by name."""
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(2):               # (the first session of a process may come up empty)
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            fn()
+            torch.cuda.synchronize()
+    out = {e.key: e.count for e in p.key_averages()}
+    if not any("dqmc" in k for k in out):
+        pytest.skip("no kernel records on this system")
+    return out
+
+
+@pytest.mark.parametrize("N,batch,fold", [(160, 64, 0), (256, 25, 0), (256, 40, 0), (256, 1, 0), (192, 2, 1)])
+def test_one_pass_per_solve(dq, N, batch, fold):
+    """The two solves of an equal-time call (N >= 160) take all instances in one pass."""
+    K, V, h = _dev(di.chain_hopping(N)), _fields(9000, batch, 6, N), dq.Handle(fold=fold)
+    runs = _kernels(lambda: dq.greens(K, 0.1, V, 3, handle=h))
+    assert sum(n for k, n in runs.items() if "solve_init_kernel" in k) == 2
+    assert sum(n for k, n in runs.items() if "lu_kernel" in k) == 0
+
+
+def test_equal_passes_above_the_cap(dq):
+    """N = 384: 512 MB hold 42 solver slots; 85 displaced points and more run in equal
+    passes, each point as by itself."""
+    N, M = 384, 4
+    K, V = _dev(di.chain_hopping(N)), _fields(9100, 20, M, N)
+    h = dq.Handle()
+    Gtt, Gt0, st = dq.greens_tdisplaced(K, 0.1, V, 1, handle=h)          # 100 points
+    assert int((st != 0).sum()) == 0
+    for b in (0, 9, 19):
+        a, c, _ = dq.greens_tdisplaced(K, 0.1, V[b], 1, handle=dq.Handle())
+        assert torch.equal(a, Gtt[b]) and torch.equal(c, Gt0[b])
