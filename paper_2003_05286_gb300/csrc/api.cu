@@ -392,7 +392,6 @@ struct TcWs {
 // N = 121 11.3 -> 11.1, N = 256 61.4 -> 55.2.
 constexpr int TC_MIN_N = 64, TC_TREE_MIN_N = 96;
 constexpr long long TC_SCRATCH = 512LL << 20;   // bytes of digits a TcWs may hold
-constexpr int TC_SHARES = 8;                    // products side by side (kMaxJobs)
 
 inline bool tc_wanted(dqmc_handle h, int N) {
   return h->lean < 1 && N >= TC_MIN_N && N <= TC_MAX_N;
@@ -425,11 +424,14 @@ void take_tc_shared(Arena& ar, int N, TcWs& w) {
   w.eEs = ar.take<int>(pad_to(N, 128));
 }
 
-void take_tc(Arena& ar, long long batch, int N, TcWs& w) {
+// Slots for `batch` instances in `shares` equal parts (tc_part) that run side by side:
+// shares - 1 slots more, so that a part holds the larger half of an odd batch, only
+// where the batch is split at all.
+void take_tc(Arena& ar, long long batch, int N, TcWs& w, int shares = 1) {
   const long long ea = tc_plane_elems(N, 128), eb = tc_plane_elems(N, 64);
   long long cap = TC_SCRATCH / (2 * (ea + eb));
-  cap = cap > 65535 ? 65535 : (cap < 1 ? 1 : cap);
-  batch += TC_SHARES - 1;                     // so that an equal share still holds its part
+  cap = cap > 65535 ? 65535 : (cap < shares ? shares : cap);
+  batch += shares - 1;
   w.cap = (int)(batch < cap ? batch : cap);
   w.A = ar.take<__nv_bfloat16>(w.cap * ea);
   w.B = ar.take<__nv_bfloat16>(w.cap * eb);
@@ -555,13 +557,15 @@ inline bool qrtc_wanted(dqmc_handle h, int N) {
   return h->lean < 1 && h->decomp == DQMC_DECOMP_QR && N >= QRTC_MIN_N && N <= QRTC_MAX_N;
 }
 
-// Slots for `batch` factorisations, and as many bytes as `solves` solves in one pass
-// take (a solver's slot holds R's digits too: N = 256 3.2 instead of 2.2 MB).
-void take_qr(Arena& ar, long long batch, int N, int row_graded, QrWs& w, long long solves) {
+// Slots for `batch` factorisations in `shares` parts (as take_tc), and as many bytes as
+// `solves` solves in one pass take (a solver's slot holds R's digits too: N = 256 3.2
+// instead of 2.2 MB).
+void take_qr(Arena& ar, long long batch, int N, int row_graded, QrWs& w, long long solves,
+             int shares = 1) {
   const long long slot = (long long)qrp_tc_slot_bytes(N, row_graded);
   long long n = TC_SCRATCH / slot;
-  batch += TC_SHARES - 1;
-  n = batch < n ? batch : (n < TC_SHARES ? TC_SHARES : n);
+  batch += shares - 1;
+  n = batch < n ? batch : (n < shares ? shares : n);
   long long bytes = n * slot;
   if (N >= SOLVETC_MIN_N) {
     const long long s = (long long)solve_tc_slot_bytes(N), m = TC_SCRATCH / s;
@@ -896,11 +900,16 @@ bool pipeline_enabled() {
 // Number of staggered sub-batches of an equal-time chain: DQMC_PIPELINE=n
 // (2..8) overrides the default of 2 (N = 256, 128 instances, 2 / 3 / 4 / 8: 128 /
 // 129 / 130 / 149 ms; reduced precision 142 / 141 / 143 / 165).
-constexpr int kMaxJobs = TC_SHARES;
+constexpr int kMaxJobs = 8;
 int pipeline_jobs() {
   const char* e = getenv("DQMC_PIPELINE");
   if (e && e[0] >= '2' && e[0] <= '8' && e[1] == 0) return e[0] - '0';
   return 2;
+}
+// Sub-batches an equal-time chain of `batch` instances runs in.
+int chain_shares(int batch) {
+  const int nj = pipeline_jobs();
+  return batch >= 4 * nj && pipeline_enabled() ? nj : 1;
 }
 
 // The jobs run on aux streams sbase .. sbase + nj - 1, forked from and joined
@@ -1653,9 +1662,10 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
       take_chain(ar, batch, N, cw);
       cw.tc = TcWs{};
       cw.qr = QrWs{};
-      if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, batch, N, cw.tc);
+      const int shares = chain_shares(batch);
+      if (tc && tc_gemms && tc_wanted(h, N)) take_tc(ar, batch, N, cw.tc, shares);
       else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, cw.tc);
-      if (tc && qrtc_wanted(h, N)) take_qr(ar, batch, N, 0, cw.qr, batch);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, batch, N, 0, cw.qr, batch, shares);
     }
     if (digits) take_ozaki(ar, batch, N, digits, cw);
     take_loh(ar, batch, N, lw);
@@ -1716,8 +1726,8 @@ static dqmc_status greens_impl(dqmc_handle h, int batch, int N, int M, const dou
     s.D = D; s.slotD = 0; s.instD = N;
     s.X = X0; s.slotX = 0; s.instX = NN;
     s.X2 = X1;
-    const int nj = pipeline_jobs();
-    if (batch >= 4 * nj && pipeline_enabled()) {
+    const int nj = chain_shares(batch);
+    if (nj > 1) {
       // nj sub-batches on nj streams, product phases staggered so that the QRs
       // of some sub-batches run while the others multiply
       ChainJob J[kMaxJobs];
@@ -2250,7 +2260,7 @@ static dqmc_status tdisplaced_impl(dqmc_handle h, int batch, int N, int M, const
       take_tc_shared(ar, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
-      take_qr(ar, Q, N, 0, cw.qr, Q);
+      take_qr(ar, batch, N, 0, cw.qr, Q);
       take_qr(ar, batch, N, 0, cw2.qr, 0);
     }
     if (const int digits = reduced_digits(h)) {
@@ -2421,7 +2431,7 @@ static dqmc_status grad_impl(dqmc_handle h, int batch, int N, int M, const doubl
       take_tc_shared(ar, N, cw2.tc);
     }
     if (tc && qrtc_wanted(h, N)) {
-      take_qr(ar, Q, N, 0, cw.qr, Q);
+      take_qr(ar, batch, N, 0, cw.qr, Q);
       take_qr(ar, batch, N, 0, cw2.qr, 0);
     }
     if (const int digits = reduced_digits(h)) {
@@ -2609,9 +2619,9 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       w.cw.tc = TcWs{};
       w.cw.qr = QrWs{};
       const int digits = reduced_digits(h);
-      if (tc && !digits && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc);
+      if (tc && !digits && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc, chain_shares(nb));
       else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, w.cw.tc);
-      if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr, nb);
+      if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr, nb, chain_shares(nb));
       if (digits) take_ozaki(ar, nb, N, digits, w.cw);
       take_loh(ar, nb, N, w.lw);
       if (h->inv == DQMC_INV_PLAIN) take_plain(ar, nb, N, w.pw);
@@ -2729,12 +2739,13 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
         sl.D = w.D; sl.slotD = 0; sl.instD = N;
         sl.X = w.X0; sl.slotX = 0; sl.instX = NN;
         sl.X2 = w.X1;
-        if (nb >= 4 * nj && pipeline_enabled()) {
+        const int shares = chain_shares(nb);
+        if (shares > 1) {
           // as a uniform call: sub-batches on their own streams, staggered so
           // that the QRs of some run while the others multiply
           ChainJob J[kMaxJobs];
-          make_sub_jobs(J, nj, +1, nb, N, w.expV, Mp * N, sl, w.cw, w.st, w.Mb);
-          CKS(run_chain_multi(h, J, nj, N, g.Mmax, k, E, (int)slot + 1));
+          make_sub_jobs(J, shares, +1, nb, N, w.expV, Mp * N, sl, w.cw, w.st, w.Mb);
+          CKS(run_chain_multi(h, J, shares, N, g.Mmax, k, E, (int)slot + 1));
         } else {
           CKS(run_chain(h, +1, nb, N, g.Mmax, k, E, w.expV, Mp * N, sl, w.cw, w.st, w.Mb));
         }

@@ -58,3 +58,30 @@ def test_equal_passes_above_the_cap(dq):
     for b in (0, 9, 19):
         a, c, _ = dq.greens_tdisplaced(K, 0.1, V[b], 1, handle=dq.Handle())
         assert torch.equal(a, Gtt[b]) and torch.equal(c, Gt0[b])
+
+
+def test_no_slots_to_spare(dq):
+    """One instance of N = 256, sequential fold: 7.1 MB of matrices, 2.1 MB of operand
+    digits, 1.1 MB of the slice matrix's, one solver slot of 3.2 MB, and the eighth a
+    workspace grows by; a displaced call has QR slots for its instances, not its points."""
+    K, V, h = _dev(di.chain_hopping(256)), _fields(9200, 1, 20, 256), dq.Handle(fold=0)
+    dq.greens(K, 0.1, V, 5, handle=h)
+    assert h.workspace_bytes <= 16 << 20
+    # N = 96, 41 points: per point 0.4 MB of digits and 16 matrices; a QR slot is 0.6 MB
+    N = 96
+    h = dq.Handle()
+    dq.greens_tdisplaced(_dev(di.chain_hopping(N)), 0.1, _fields(9300, 1, 40, N), 1, handle=h)
+    assert h.workspace_bytes <= 9 / 8 * 41 * (0.4e6 + 22 * 8 * N * N) + (6 << 20)
+
+
+@pytest.mark.parametrize("jobs,batch", [("2", 9), ("3", 13), ("8", 33), ("8", 39)])
+def test_odd_shares(dq, monkeypatch, jobs, batch):
+    """Batches that split unevenly into sub-batches: every instance as by itself."""
+    N = 160
+    K, V = _dev(di.chain_hopping(N)), _fields(9400, batch, 8, N)
+    one = [dq.greens(K, 0.1, V[b], 4, handle=dq.Handle(fold=0)) for b in range(batch)]
+    monkeypatch.setenv("DQMC_PIPELINE", jobs)
+    G, ld, sg, st = dq.greens(K, 0.1, V, 4, handle=dq.Handle(fold=0))
+    assert int((st != 0).sum()) == 0
+    for b in range(batch):
+        assert torch.equal(G[b], one[b][0]) and float(ld[b]) == float(one[b][1])
