@@ -2599,10 +2599,31 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
     if (d.M > g->Mmax) g->Mmax = d.M;
   }
   // ---- workspace (h->ws) and index tables (h->rtab): one region per group ----
+  // Up to 8 groups run side by side, group i in stream slot i % nslots; those of a slot
+  // run one after another and share its scratch for the tensor-core kernels (a batch of
+  // distinct matrices has one group per instance).
+  const size_t nslots = groups.size() < 8 ? groups.size() : 8;
   std::vector<RaggedGroupWs> gw(groups.size());
   int lean = 0;
+  auto scratch = [&](Arena& ar, const RaggedGroup& g, ChainWs& w) {
+    const int nb = (int)g.idx.size(), N = g.N, shares = chain_shares(nb);
+    w.tc = TcWs{};
+    w.qr = QrWs{};
+    if (lean >= 1) return;
+    if (!reduced_digits(h) && tc_wanted(h, N)) take_tc(ar, nb, N, w.tc, shares);
+    else if (!reduced_digits(h) && chain_tc_wanted(h, N)) take_tc_shared(ar, N, w.tc);
+    if (qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.qr, nb, shares);
+  };
   auto layout = [&](Arena& ar) {
-    const bool tc = lean < 1;
+    std::vector<size_t> need(nslots, 0);
+    for (size_t i = 0; i < groups.size(); ++i) {
+      Arena m;
+      scratch(m, groups[i], gw[i].cw);
+      need[i % nslots] = std::max(need[i % nslots], m.off);
+    }
+    std::vector<char*> slot_ws(nslots, nullptr);
+    for (size_t q = 0; q < nslots; ++q)
+      if (need[q]) slot_ws[q] = ar.take<char>((long long)need[q]);
     for (size_t i = 0; i < groups.size(); ++i) {
       const RaggedGroup& g = groups[i];
       RaggedGroupWs& w = gw[i];
@@ -2616,13 +2637,10 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
       w.X0 = ar.take<double>(NN * nb);
       w.X1 = ar.take<double>(NN * nb);
       take_chain(ar, nb, N, w.cw);
-      w.cw.tc = TcWs{};
-      w.cw.qr = QrWs{};
-      const int digits = reduced_digits(h);
-      if (tc && !digits && tc_wanted(h, N)) take_tc(ar, nb, N, w.cw.tc, chain_shares(nb));
-      else if (tc && !digits && chain_tc_wanted(h, N)) take_tc_shared(ar, N, w.cw.tc);
-      if (tc && qrtc_wanted(h, N)) take_qr(ar, nb, N, 0, w.cw.qr, nb, chain_shares(nb));
-      if (digits) take_ozaki(ar, nb, N, digits, w.cw);
+      Arena sub;
+      sub.base = slot_ws[i % nslots];
+      scratch(sub, g, w.cw);
+      if (const int digits = reduced_digits(h)) take_ozaki(ar, nb, N, digits, w.cw);
       take_loh(ar, nb, N, w.lw);
       if (h->inv == DQMC_INV_PLAIN) take_plain(ar, nb, N, w.pw);
       w.G = ar.take<double>(NN * nb);
@@ -2688,10 +2706,9 @@ static dqmc_status ragged_impl(dqmc_handle h, int batch, const dqmc_instance* de
     h->rtab_key = dkey;
   }
   // ---- streams and the fork event (created outside any capture) --------------
-  // up to 8 group slots; a slot has its group's stream and nj more for the
-  // staggered sub-batches of a group large enough to pipeline
+  // a slot has its group's stream and nj more for the staggered sub-batches of a
+  // group large enough to pipeline
   const int nj = pipeline_jobs();
-  const size_t nslots = groups.size() < 8 ? groups.size() : 8;
   const size_t per_slot = (size_t)nj + 1;
   const size_t nstreams = nslots * per_slot;
   CKS(ensure_aux(h, nstreams));

@@ -85,3 +85,31 @@ def test_odd_shares(dq, monkeypatch, jobs, batch):
     assert int((st != 0).sum()) == 0
     for b in range(batch):
         assert torch.equal(G[b], one[b][0]) and float(ld[b]) == float(one[b][1])
+
+
+def test_ragged_groups_share_scratch(dq):
+    """24 instances with a K of their own are 24 groups, of which 8 run side by side: those
+    past the eighth add their matrices (15 to 18 of N x N), but no digits and no QR slot
+    (1.2 MB at N = 96, 16 matrices).  Every instance equals its own call bitwise, also
+    among groups of other sizes."""
+    N, M = 96, 12
+    insts = [(_dev(di.chain_hopping(N)), 0.1, V, 4) for V in _fields(9500, 24, M, N)]
+    held = []
+    for n in (8, 24):
+        h = dq.Handle()
+        dq.greens_ragged(insts[:n], handle=h)
+        held.append(h.workspace_bytes)
+    assert held[1] - held[0] <= 9 / 8 * 16 * 18 * 8 * N * N
+    sizes = [40, 64, 64, 96, 130, 160, 200, 64, 256, 33, 96, 48, 160, 20, 64, 300, 72, 100, 64, 161]
+    mix = [(_dev(di.chain_hopping(n)), 0.1, _fields(9600 + i, 1, M, n)[0], 4) for i, n in enumerate(sizes)]
+    K = _dev(di.chain_hopping(128))
+    mix += [(K, 0.1, V, 4) for V in _fields(9700, 11, M, 128)]           # one group, two sub-batches
+    for todo in (insts, mix):
+        for graphs in (False, True):
+            hg = dq.Handle(graphs=graphs)
+            for _ in range(2):
+                G, ld, sg, st = dq.greens_ragged(todo, handle=hg)
+            assert int((st != 0).sum()) == 0
+            for i, (K1, dt, V1, k) in enumerate(todo):
+                G1, ld1, _, _ = dq.greens(K1, dt, V1, k, handle=dq.Handle(fold=0))
+                assert torch.equal(G1, G[i]) and float(ld1) == float(ld[i])
