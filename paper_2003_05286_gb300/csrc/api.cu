@@ -122,7 +122,10 @@ bool within_limit(dqmc_handle h, size_t old, size_t bytes) {
   return h->mem_limit == 0 || held_bytes(h) - old + bytes <= h->mem_limit;
 }
 
-dqmc_status ensure_ws(dqmc_handle h, size_t bytes) {
+// spare: the caller goes on with a smaller layout when there is no room.  The buffer is
+// then only given back for one that the device's free memory can hold, so that calls on
+// a full device keep the smaller workspace instead of replacing it each time.
+dqmc_status ensure_ws(dqmc_handle h, size_t bytes, bool spare = false) {
   if (bytes <= h->ws_bytes) return DQMC_OK;
   if (h->capturing) {   // no allocation inside a capture: the caller grows and captures again
     h->ws_need = bytes;
@@ -131,6 +134,11 @@ dqmc_status ensure_ws(dqmc_handle h, size_t bytes) {
   if (!within_limit(h, h->ws_bytes, bytes)) return DQMC_ERR_NOMEM;
   size_t want = bytes + bytes / 8;
   if (!within_limit(h, h->ws_bytes, want)) want = bytes;
+  if (spare) {
+    size_t room = 0, total = 0;
+    if (cudaMemGetInfo(&room, &total) != cudaSuccess) return DQMC_ERR_CUDA;
+    if (bytes > room + h->ws_bytes) return DQMC_ERR_NOMEM;
+  }
   h->gvalid = false;    // a captured graph refers to the old workspace
   if (h->ws) {
     cudaStreamSynchronize(h->stream);
@@ -164,9 +172,10 @@ dqmc_status place(dqmc_handle h, int& lean, F&& layout) {
   while (true) {
     Arena measure;
     layout(measure);
-    const dqmc_status rc = ensure_ws(h, measure.off);
+    const bool spare = lean < max_lean(h);
+    const dqmc_status rc = ensure_ws(h, measure.off, spare);
     if (rc == DQMC_OK) break;
-    if (rc != DQMC_ERR_NOMEM || h->capturing || lean >= max_lean(h)) return rc;
+    if (rc != DQMC_ERR_NOMEM || h->capturing || !spare) return rc;
     ++lean;
   }
   Arena ar;
@@ -1570,9 +1579,10 @@ static dqmc_status graph_call(dqmc_handle h, GraphKey key, F&& body) {
     if (rc == DQMC_ERR_NOMEM && h->ws_need) {   // grow outside the capture, then record again
       if (g) cudaGraphDestroy(g);
       cudaGetLastError();
-      const dqmc_status grown = ensure_ws(h, h->ws_need);
+      const bool spare = h->lean < max_lean(h);
+      const dqmc_status grown = ensure_ws(h, h->ws_need, spare);
       if (grown != DQMC_OK) {
-        if (grown != DQMC_ERR_NOMEM || h->lean >= max_lean(h)) return grown;
+        if (grown != DQMC_ERR_NOMEM || !spare) return grown;
         ++h->lean;   // record again with less
         continue;
       }

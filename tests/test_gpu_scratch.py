@@ -113,3 +113,39 @@ def test_ragged_groups_share_scratch(dq):
             for i, (K1, dt, V1, k) in enumerate(todo):
                 G1, ld1, _, _ = dq.greens(K1, dt, V1, k, handle=dq.Handle(fold=0))
                 assert torch.equal(G1, G[i]) and float(ld1) == float(ld[i])
+
+
+@pytest.mark.parametrize("graphs", [False, True])
+def test_full_device_keeps_the_workspace(dq, graphs):
+    """128 instances of N = 256 on a device with 300 MB too little for the whole workspace
+    (0.7 GB of digits beside 0.9 GB of matrices).  The calls run without the digits, and after the first one none of them
+    allocates or frees device memory."""
+    from torch.profiler import ProfilerActivity, profile
+    N, M, batch = 256, 4, 128
+    K, V = _dev(di.chain_hopping(N)), _fields(9800, batch, M, N)
+    h0 = dq.Handle(fold=0)
+    ref = dq.logdet(K, 0.1, V, 2, handle=h0)
+    full = h0.workspace_bytes
+    h0.close()
+    h = dq.Handle(fold=0, graphs=graphs)
+    dq.logdet(K, 0.1, V[:1], 2, handle=h)          # loads the kernels
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    room = full * 8 // 9 - (300 << 20)             # too little for the digits by 300 MB
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+    try:
+        ld, sg, st = dq.logdet(K, 0.1, V, 2, handle=h)
+        held = h.workspace_bytes
+        assert held < room and int((st != 0).sum()) == 0
+        for _ in range(2):
+            with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as p:
+                ld, sg, st = dq.logdet(K, 0.1, V, 2, handle=h)
+                torch.cuda.synchronize()
+        names = {e.key for e in p.key_averages()}
+        assert any("cuda" in n for n in names)
+        assert not names & {"cudaFree", "cudaMalloc"}
+        assert h.workspace_bytes == held
+        assert ((ld - ref[0]).abs() <= 1e-9 * ref[0].abs()).all() and torch.equal(sg, ref[1])
+    finally:
+        del fill
+        torch.cuda.empty_cache()
