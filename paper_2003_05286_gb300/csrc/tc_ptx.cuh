@@ -103,7 +103,7 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// (T 2^32 + r) 2^e correctly rounded to FP64, for |T| < 2^62 and 0 <= r < 2^32
+// (T 2^32 + r) 2^e correctly rounded to FP64 (subnormal results too), for |T| < 2^62 and 0 <= r < 2^32
 // (the exact sum of the weight groups), with 32-bit integer operations and no
 // branch but for results outside the normal range: the FP64 pipe stays free, and
 // a CTA's epilogue converts thousands of sums.  The magnitude's three words are
@@ -135,8 +135,18 @@ __host__ __device__ __forceinline__ double split_times_pow2(long long T, unsigne
                             (unsigned long long)((m1 << 21) | (m0 >> 11)) + up;
   bits |= (unsigned long long)neg << 63;
   if (w2 == 0u) bits = 0ull;
-  else if (be < 1 || be > 2044)              // result outside the normal range: scale in FP64
-    return ldexp((double)Tm * 4294967296.0 + (double)w0n, e) * (neg ? -1.0 : 1.0);
+  else if (be < 0 || be > 2045) {            // result outside the normal range
+    const unsigned long long m = ((unsigned long long)m1 << 32) | m0;
+    const int sh = 11 - be;                  // the last bit kept is 2^-1074
+    if (be > 0) bits = 0x7ffull << 52;
+    else if (sh > 64) bits = 0ull;
+    else {
+      const unsigned long long half = 1ull << (sh - 1), rem = sh < 64 ? m & (2 * half - 1) : m;
+      bits = sh < 64 ? m >> sh : 0ull;
+      bits += rem > half || (rem == half && (low || (bits & 1ull))) ? 1u : 0u;
+    }
+    bits |= (unsigned long long)neg << 63;
+  }
 #ifdef __CUDA_ARCH__
   return __longlong_as_double((long long)bits);
 #else
