@@ -261,36 +261,6 @@ __device__ __noinline__ void pivot_search(const double* W, const double* Din, co
   }
 }
 
-// nrm = sqrt(sig) and gam = 1 / (sig + |alpha| nrm) for a normal sig > 0, |alpha| <=
-// nrm (1 + eps): the library's square root and division are chains of some 20 FP64
-// instructions on one warp, each holding the pipe for 64 cycles, with every other
-// warp waiting.  FP32 seeds (22 bits, scaled by exponent arithmetic) and FP64
-// corrections take 9 in a row: one Goldschmidt step and Markstein's residual
-// correction for the root (P. Markstein, IBM J. Res. Dev. 34, 1990), one cubic
-// Newton step for the reciprocal.  Checked against long double over 2e7 random
-// arguments: the root is the correctly rounded one, gam within 1.93 units of
-// 2^-53 (1.90 with IEEE operations).  32 steps on 32 rows: 106 -> 98 thousand cycles.
-__device__ __forceinline__ void norm_and_gamma(double sig, double alpha, double& nrm, double& gam) {
-  const long long sb = __double_as_longlong(sig);
-  const int ex = (int)(sb >> 52) - 1023, half = ex >> 1;
-  const float m = __uint_as_float(((uint32_t)(127 + (ex & 1)) << 23) | (uint32_t)((sb >> 29) & 0x7fffff));
-  const uint32_t yu = __float_as_uint(rsqrtf(m));
-  const double y0 = __longlong_as_double(((long long)((int)(yu >> 23) - 127 + 1023 - half) << 52) |
-                                         ((long long)(yu & 0x7fffff) << 29));
-  const double g0 = sig * y0, h0 = 0.5 * y0, r0 = fma(-g0, h0, 0.5);
-  const double g1 = fma(g0, r0, g0), h1 = fma(h0, r0, h0);
-  nrm = fma(fma(-g1, g1, sig), h1, g1);
-  const double D = fma(fabs(alpha), nrm, sig);
-  const long long db = __double_as_longlong(D);
-  const int de = (int)(db >> 52) - 1023;
-  const uint32_t zu = __float_as_uint(
-      __fdividef(1.0f, __uint_as_float((127u << 23) | (uint32_t)((db >> 29) & 0x7fffff))));
-  const double z0 = __longlong_as_double(((long long)((int)(zu >> 23) - 127 + 1023 - de) << 52) |
-                                         ((long long)(zu & 0x7fffff) << 29));
-  const double e = fma(-D, z0, 1.0);
-  gam = fma(z0, fma(e, e, e), z0);
-}
-
 // FP64 Householder reduction of the chosen columns by the first LPC warps, LPC
 // lanes a column (row l + LPC k in register k).  Every FP64 warp instruction
 // holds its sub-partition's pipe for 64 cycles: short panels take 8 lanes (few
