@@ -42,10 +42,12 @@
 // is.  When the rows of A are graded too (Drow: the levels of the tree fold, whose
 // factor D_2 sits on the left), Householder QR with column pivoting is accurate
 // row by row (Cox and Higham, 1998), and so must be the update of A: it then uses
-// a second set of digits of the unnormalised u, where u_rj has the size s_r of
-// row r.  V W2 has row exponents (W2 is of order one), and V^T A multiplies
-// 2^{rho_r} u_rj by 2^{-rho_r} a_rc, 2^{rho_r} ~ s_r = Drow_r, so that both
-// factors' largest entries meet in the same row.  Q needs only the first set.
+// a second set of digits in which u_rj has the size s_r of row r: V W2 has row
+// exponents, its columns u_j 2^{-h_j} with max_r u_rj 2^{-rho_r - h_j} of order one,
+// 2^{rho_r} ~ s_r = Drow_r (a pivot column that D_1 puts in front of larger ones would
+// otherwise meet the others' W2 at its own size), and V^T A multiplies 2^{rho_r} u_rj
+// by 2^{-rho_r} a_rc, so that both factors' largest entries meet in the same row.  Q
+// needs only the first set.
 // T is the first set's in both (the scales go in and out as exponents), so that
 // nothing squares a column's scale: norms over FP64's whole range are taken.
 #include <cuda_bf16.h>
@@ -477,7 +479,7 @@ struct QrTc {
   unsigned char* ws;         // per slot: see the pointers below
   long long slot_bytes;
   __host__ __device__ long long set_bytes() const {
-    return (long long)np * (nkb * VT_TILE + nmt * V_TILE + NB * NB * 8 + NB * 4 + 32 * nkb * 4);
+    return (long long)np * (nkb * VT_TILE + nmt * V_TILE + NB * NB * 8 + 2 * NB * 4 + 32 * nkb * 4);
   }
   __host__ __device__ unsigned char* slot(int z) const { return ws + (long long)z * slot_bytes; }
   __host__ __device__ unsigned char* vt(int z, int p, int set) const {   // V^T tiles of panel p
@@ -490,13 +492,14 @@ struct QrTc {
     return reinterpret_cast<double*>(v(z, np, set)) + p * (NB * NB);
   }
   // exponents: f_j of V^T's rows (in the first set the scales of its vectors), in the
-  // second set also e_r of V's rows
+  // second set also e_r of V's rows and h_j of its columns
   __host__ __device__ int* f(int z, int p, int set) const {
     return reinterpret_cast<int*>(T(z, np, set)) + p * NB;
   }
   __host__ __device__ int* er(int z, int p, int set) const {
     return f(z, np, set) + p * 32 * nkb;
   }
+  __host__ __device__ int* h(int z, int p, int set) const { return er(z, np, set) + p * NB; }
   // the column scales, kept here because D may be written over Din
   __host__ __device__ double* din(int z) const {
     return reinterpret_cast<double*>(slot(z) + sets * set_bytes());
@@ -737,16 +740,7 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   for (int set = 0; set < a.sets; ++set) {
     // ---- exponents: first set of the columns alone, second set with the row scales and
     // of the rows ---------------------------------------------------------------------
-    if (tid < 32 * nkl) {
-      if (set) {
-        int mx = 0;
-        for (int c = 0; c < NB; ++c)
-          mx = max(mx, (int)((__double_as_longlong(us[c * LDU + tid]) >> 52) & 0x7ff));
-        s_er[tid] = mx == 0x7ff ? 0 : tc_exponent(mx);
-        a.er(z, p, 1)[j0 + tid] = s_er[tid];
-      }
-      s_rho[tid] = set ? row_rho(Drow, j0 + tid, N) : 0;
-    }
+    if (tid < 32 * nkl) s_rho[tid] = set ? row_rho(Drow, j0 + tid, N) : 0;
     __syncthreads();
     {
       const int c = tid >> 4, l = tid & 15;
@@ -770,7 +764,18 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
         s_h[c] = bad ? TC_NONFINITE : (mf == 0 ? 0 : mh - 1020);
         if (!set) s_f0[c] = s_f[c];
         a.f(z, p, set)[c] = s_f[c];
+        if (set) a.h(z, p, 1)[c] = s_h[c];
       }
+    }
+    __syncthreads();
+    if (set && tid < 32 * nkl) {            // (NaN and inf come in with f_j)
+      int mx = 0;
+      for (int c = 0; c < NB; ++c) {
+        const int E = (int)((__double_as_longlong(us[c * LDU + tid]) >> 52) & 0x7ff);
+        if (E != 0 && E != 0x7ff && s_h[c] < TC_NONFINITE / 2) mx = max(mx, E - s_h[c] + 100000);
+      }
+      s_er[tid] = mx == 0 ? 0 : mx - 100000 - 1020;
+      a.er(z, p, 1)[j0 + tid] = s_er[tid];
     }
     __syncthreads();
     // ---- digits of V^T (to the tiles and the staging ring) and V^T V: four 32-row
@@ -814,7 +819,7 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
       unsigned char* gv = a.v(z, p, set) + (long long)t * V_TILE;
       const int rr = tid >> 2, ch = tid & 3, r = 128 * t + rr - j0;
       const int er = set && r >= 0 && r < m ? s_er[r] : 0;
-      tc_digits<8>([&](int k) { return set ? er : s_f[8 * ch + k]; },
+      tc_digits<8>([&](int k) { return set ? er + s_h[8 * ch + k] : s_f[8 * ch + k]; },
                    [&](int k) { return r >= 0 && r < m ? us[(8 * ch + k) * LDU + r] : 0.0; },
                    [&](int q, const uint32_t (&w)[4]) {
                      *reinterpret_cast<uint4*>(gv + q * (128 * 64) + swz(rr, ch)) =
@@ -916,7 +921,7 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
   int* ew = ecol + 32;
   int* s_f = ew + 32;                                           // [32]
   int* s_f0 = s_f + 32;                                         // [32]
-  double* s_dn = reinterpret_cast<double*>(s_f0 + 32);          // [32] 2^{-f0}
+  double* s_dn = reinterpret_cast<double*>(s_f0 + 32);          // [32] 2^{h - f0}
   int* s_rho = reinterpret_cast<int*>(s_dn + 32);               // [32 nkb]
   int* s_er = s_rho + 32 * a.nkb;                               // [32 nkb]
   uint64_t* full = reinterpret_cast<uint64_t*>(s_er + 32 * a.nkb);
@@ -984,7 +989,7 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
       ew[tid] = 0;
       s_f[tid] = set ? a.f(z, pp, 1)[tid] : 0;
       s_f0[tid] = set ? a.f(z, pp, 0)[tid] : 0;
-      s_dn[tid] = set ? scalbn(1.0, -s_f0[tid]) : 1.0;
+      s_dn[tid] = set ? scalbn(1.0, a.h(z, pp, 1)[tid] - s_f0[tid]) : 1.0;
     }
     for (int r = tid; r < 32 * a.nkb; r += 512) {
       s_rho[r] = set ? row_rho(Drow, r, N) : 0;
@@ -1079,7 +1084,7 @@ __global__ void __launch_bounds__(512, 1) qr_apply_kernel(const QrTc a, int p) {
           if (l <= i) s0 = fma(tt[l * TLD + i], w1[l * TLD + lane], s0);
         }
         double s = s0 + s1;
-        if (set) s *= s_dn[i];               // V's digits are those of u itself
+        if (set) s *= s_dn[i];               // V's digits are those of u_i 2^{-h_i}
         w2[i * TLD + lane] = s;
         atomicMax(&ew[lane], (int)((__double_as_longlong(s) >> 52) & 0x7ff));
       }
