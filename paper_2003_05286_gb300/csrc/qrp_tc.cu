@@ -36,8 +36,13 @@
 // panel 255 (the FP64 pipe, plus a square root, a division and two barriers per
 // column), digits and V^T V 27, T 12; an apply of 256 rows 55.
 //
-// V's columns are scaled by powers of two into (-1/4, 1/4) (|u_r| <= |u_j|), so
-// V needs no exponents and T takes up the scales: every product is then accurate
+// V's columns are v_j = u_j / u_jj, H_j = 1 - tau_j v_j v_j^T with tau_j = (beta_j -
+// alpha_j) / beta_j.  A column that is a multiple of a unit vector then gives exact
+// digits, T and Q, and decoupled sites stay decoupled.  (With u_j scaled by powers of two
+// alone the rounding of gamma put 2^-53 into Q's zeros, times the grading of the next
+// chunk: K = 0, fields of variance 4, N = 160, M = 40, k = 10, error of G 6e-8 -> 1e-15;
+// one N = 256 factorisation takes 1.5% longer.)  |v_r| <= 1 = v_j, so V needs no
+// exponents and T takes up the scales: every product is then accurate
 // column by column against the column's largest entry, as Householder's method
 // is.  When the rows of A are graded too (Drow: the levels of the tree fold, whose
 // factor D_2 sits on the left), Householder QR with column pivoting is accurate
@@ -268,8 +273,9 @@ __device__ __noinline__ void pivot_search(const double* W, const double* Din, co
 // holds its sub-partition's pipe for 64 cycles: short panels take 8 lanes (few
 // reduction levels, few warps), tall ones 16 (the columns left spread evenly
 // over the sub-partitions; N = 256, 32 columns: 323 -> 240 thousand cycles).  A
-// warp whose columns are done drops out.  Leaves R in W^T and u_j (zeros above j)
-// in out[0]; out[1]: two columns of workspace.
+// warp whose columns are done drops out.  Leaves R in W^T and in out[0] v_j 2^{E_j}, v_j =
+// u_j / u_jj (zeros above j), with tau_j = (beta_j - alpha_j) / beta_j, H_j = 1 - tau_j v_j
+// v_j^T, in s_beta (0 for H_j = 1) and E_j in s_ex; out[1]: two columns of workspace.
 // s_gam[j] is the gamma of u_j 2^{-s_ex[j]}.  Squares of the columns as they are
 // (s_ex = 0) serve while they stay inside FP64's range.  Where one of a panel's steps
 // met one outside (gamma is left at zero) the first form returns true and writes
@@ -363,14 +369,32 @@ __device__ __noinline__ bool panel_factor(double* W, const int* s_rem, const int
   }
   // (written before the last barrier of the loop: every warp sees the same)
   if (!WIDE && __any_sync(FULL, lane < nb && s_gam[lane] == 0.0)) return true;
+  // u_j is left as v_j 2^{E_j}: the leading entry, and one as large, exactly +-2^{E_j}
   const double up = WIDE && own ? scalbn(1.0, s_ex[pc]) : 1.0;
+  const bool on = own && s_gam[pc] > 0.0;
+  const double beta = own ? s_beta[pc] : 0.0, uj = on ? s_uj[pc] : 1.0, u = WIDE ? uj * up : uj;
+  const long long ub = __double_as_longlong(u), top = 0x7ffll << 52;
+  const double mant = __longlong_as_double((ub & ~top) | (1023ll << 52));
+  const double mu = copysign(recip_newton(fabs(mant)), mant);
+  const double b1 = on ? fabs(beta) : 1.0, zb = recip_newton(b1);
+  double tau = fabs(uj) * zb;
+  tau = fma(fma(-tau, b1, fabs(uj)), zb, tau);
 #pragma unroll
   for (int k = 0; k < KR; ++k) {
     const int r = l8 + LPC * k;
     if (r < rows) {
-      us[r] = own && r < m && r >= pc && s_gam[pc] > 0.0 ? (r == pc ? (WIDE ? s_uj[pc] * up : s_uj[pc]) : x[k]) : 0.0;
-      if (own && r <= pc && r < m) col[r] = r == pc ? (WIDE ? s_beta[pc] * up : s_beta[pc]) : x[k];
+      const double xr = r == pc ? u : x[k];
+      const long long xb = __double_as_longlong(xr) ^ ub;
+      us[r] = on && r < m && r >= pc
+                  ? ((xb << 1) == 0 ? __longlong_as_double((ub & top) | (xb & (1ll << 63))) : xr * mu)
+                  : 0.0;
+      if (own && r <= pc && r < m) col[r] = r == pc ? (WIDE ? beta * up : beta) : x[k];
     }
+  }
+  __syncwarp();
+  if (l8 == 0) {
+    s_beta[pc] = on ? tau : 0.0;
+    s_ex[pc] = (int)((ub & top) >> 52) - 1023;
   }
   return false;
 }
@@ -603,7 +627,7 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   int* s_rem = reinterpret_cast<int*>(s_key + N);              // [m]
   int* s_cand = s_rem + N;                                     // [CN] positions in rem
   int* s_sel = s_cand + CN;                                    // [32] candidate numbers
-  int* s_ex = s_sel + NB;                                      // [32] exponents of gamma's vectors
+  int* s_ex = s_sel + NB;                                      // [32] E_j (panel_factor)
   int* s_f0 = s_ex + NB;                                       // [32] the first set's s_f
   int* s_f = s_f0 + NB;                                        // [32] exponents of V^T's rows
   int* s_h = s_f + NB;                                         // [32] of V's columns times 2^{-rho_r}
@@ -736,6 +760,8 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   }
 #undef DQMC_FACTOR
   __syncthreads();
+  double* s_tau = s_beta;                   // (panel_factor's last step)
+  int* s_E = s_ex;
   uint32_t nm = 0;                          // MMA groups waited for
   for (int set = 0; set < a.sets; ++set) {
     // ---- exponents: first set of the columns alone, second set with the row scales and
@@ -840,12 +866,12 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
       const int i = e & 31, c = e >> 5;
       gm[i * TLD + c] = stacked_value(ex, i, c, set ? s_h[i] + s_f[c] - s_f0[i] - s_f0[c] : 0);
     }
-    double* s_g = xs;                       // (xs is free) gamma_j 2^{2 f_j}
+    double* s_g = xs;                       // (xs is free) tau_j 2^{2 (f_j - E_j)}
     if (!set && tid < NB)
-      s_g[tid] = tid < nb && s_f[tid] < TC_NONFINITE / 2 ? scalbn(s_gam[tid], 2 * (s_f[tid] - s_ex[tid])) : 0.0;
+      s_g[tid] = s_f[tid] < TC_NONFINITE / 2 ? scalbn(s_tau[tid], 2 * (s_f[tid] - s_E[tid])) : 0.0;
     for (int e = tid; e < NB * TLD; e += 512) tm[e] = 0.0;
     __syncthreads();
-    // ---- T: T_jj = gamma_j, T(:j, j) = -gamma_j T(:j,:j) G(:j, j); 8 x 8 blocks by one
+    // ---- T: T_jj = tau_j, T(:j, j) = -tau_j T(:j,:j) G(:j, j); 8 x 8 blocks by one
     // warp each, then T12 = -T11 (G12 T22) twice ---------------------------------------
     if (wid < 4 && lane < 8) {
       const int o = 8 * wid;

@@ -157,6 +157,19 @@ __host__ __device__ __forceinline__ double split_times_pow2(long long T, unsigne
 #endif
 }
 
+// 1 / D for a normal D > 0 whose reciprocal is normal, within 2 units of 2^-53: an FP32
+// seed (22 bits, scaled by exponent arithmetic) and one cubic Newton step.
+__device__ __forceinline__ double recip_newton(double D) {
+  const long long db = __double_as_longlong(D);
+  const int de = (int)(db >> 52) - 1023;
+  const uint32_t zu = __float_as_uint(
+      __fdividef(1.0f, __uint_as_float((127u << 23) | (uint32_t)((db >> 29) & 0x7fffff))));
+  const double z0 = __longlong_as_double(((long long)((int)(zu >> 23) - 127 + 1023 - de) << 52) |
+                                         ((long long)(zu & 0x7fffff) << 29));
+  const double e = fma(-D, z0, 1.0);
+  return fma(z0, fma(e, e, e), z0);
+}
+
 // nrm = sqrt(sig) and gam = 1 / (sig + |alpha| nrm) for a normal sig > 0, |alpha| <=
 // nrm (1 + eps): the library's square root and division are chains of some 20 FP64
 // instructions on one warp, each holding the pipe for 64 cycles, with every other
@@ -176,15 +189,7 @@ __device__ __forceinline__ void norm_and_gamma(double sig, double alpha, double&
   const double g0 = sig * y0, h0 = 0.5 * y0, r0 = fma(-g0, h0, 0.5);
   const double g1 = fma(g0, r0, g0), h1 = fma(h0, r0, h0);
   nrm = fma(fma(-g1, g1, sig), h1, g1);
-  const double D = fma(fabs(alpha), nrm, sig);
-  const long long db = __double_as_longlong(D);
-  const int de = (int)(db >> 52) - 1023;
-  const uint32_t zu = __float_as_uint(
-      __fdividef(1.0f, __uint_as_float((127u << 23) | (uint32_t)((db >> 29) & 0x7fffff))));
-  const double z0 = __longlong_as_double(((long long)((int)(zu >> 23) - 127 + 1023 - de) << 52) |
-                                         ((long long)(zu & 0x7fffff) << 29));
-  const double e = fma(-D, z0, 1.0);
-  gam = fma(z0, fma(e, e, e), z0);
+  gam = recip_newton(fma(fabs(alpha), nrm, sig));
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {

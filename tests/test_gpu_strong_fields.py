@@ -78,3 +78,49 @@ def test_tree_of_weakly_coupled_sites(dq, N, seed, k):
     assert int(st) == 0 and int(sg) == 1
     assert np.abs(G.cpu().numpy() - Gx).max() <= GTOL
     assert abs(float(ld) - ldx) <= LTOL * max(1.0, abs(ldx))
+
+
+def _sites(kind, N):
+    return np.zeros(N) if kind == "alike" else np.linspace(-3.0, 3.0, N)
+
+
+@pytest.mark.parametrize("k", [5, 10])
+@pytest.mark.parametrize("kind", ["alike", "levels"])
+@pytest.mark.parametrize("N", [48, 64, 100, 160, 257])
+def test_sites_alone(dq, N, kind, k):
+    """K diagonal: every site is its own problem, whatever the others' fields (factors e^{+-30}
+    of each other in one chunk).  G = 1 / (1 + e^{s}) with s a sum of M terms of order one: a
+    few M rounding errors of 2^-53 each."""
+    M, K = 40, _sites(kind, N)
+    tol = 4 * M * 2.0 ** -53
+    V = 2.0 * np.random.default_rng(100 * N).standard_normal((2, M, N))
+    sums = V.sum(1) - 0.1 * M * K
+    g, h = 1.0 / (1.0 + np.exp(sums)), dq.Handle(fold=0)
+    Kd, Vd = _dev(np.diag(K)), _dev(V)
+    G, ld, sg, st = dq.greens(Kd, 0.1, Vd, k, handle=h)
+    assert int((st != 0).sum()) == 0 and int((sg != 1).sum()) == 0
+    G = G.cpu().numpy()
+    for b in range(2):
+        assert np.abs(G[b] - np.diag(g[b])).max() <= tol
+        want = np.log1p(np.exp(sums[b])).sum()
+        assert abs(float(ld[b]) - want) <= tol * (1.0 + np.abs(sums[b])).sum()
+    _, Gt0, st = dq.greens_tdisplaced(Kd, 0.1, Vd, k, want_tt=False)
+    assert int((st != 0).sum()) == 0
+    for b in range(2):
+        for j in range(Gt0.shape[1]):
+            t0 = np.exp(V[b, : j * k].sum(0) - 0.1 * j * k * K) * g[b]
+            assert np.abs(Gt0[b, j].cpu().numpy() - np.diag(t0)).max() <= tol * max(1.0, t0.max())
+
+
+@pytest.mark.parametrize("k", [5, 10])
+@pytest.mark.parametrize("N", [64, 160])
+def test_sites_alone_tree(dq, N, k):
+    """The same in the tree fold, whose factors are graded on both sides; the suite's tolerance."""
+    V = np.stack([_ising(N, 40, 1.2, 100 * N + s) for s in range(4)])
+    s = V.sum(1)
+    G, ld, sg, st = dq.greens(_dev(np.zeros((N, N))), 0.1, _dev(V), k, handle=dq.Handle(fold=1))
+    assert int((st != 0).sum()) == 0
+    for b in range(4):
+        assert np.abs(G[b].cpu().numpy() - np.diag(1.0 / (1.0 + np.exp(s[b])))).max() <= GTOL
+        want = np.log1p(np.exp(s[b])).sum()
+        assert abs(float(ld[b]) - want) <= LTOL * max(1.0, want)
