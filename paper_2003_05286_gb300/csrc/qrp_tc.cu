@@ -41,7 +41,7 @@
 // digits, T and Q, and decoupled sites stay decoupled.  (With u_j scaled by powers of two
 // alone the rounding of gamma put 2^-53 into Q's zeros, times the grading of the next
 // chunk: K = 0, fields of variance 4, N = 160, M = 40, k = 10, error of G 6e-8 -> 1e-15;
-// one N = 256 factorisation takes 1.5% longer.)  |v_r| <= 1 = v_j, so V needs no
+// one N = 256 factorisation 1.618 -> 1.626 ms.)  |v_r| <= 1 = v_j, so V needs no
 // exponents and T takes up the scales: every product is then accurate
 // column by column against the column's largest entry, as Householder's method
 // is.  When the rows of A are graded too (Drow: the levels of the tree fold, whose
@@ -274,8 +274,7 @@ __device__ __noinline__ void pivot_search(const double* W, const double* Din, co
 // reduction levels, few warps), tall ones 16 (the columns left spread evenly
 // over the sub-partitions; N = 256, 32 columns: 323 -> 240 thousand cycles).  A
 // warp whose columns are done drops out.  Leaves R in W^T and in out[0] v_j 2^{E_j}, v_j =
-// u_j / u_jj (zeros above j), with tau_j = (beta_j - alpha_j) / beta_j, H_j = 1 - tau_j v_j
-// v_j^T, in s_beta (0 for H_j = 1) and E_j in s_ex; out[1]: two columns of workspace.
+// u_j / u_jj, 2^{E_j} <= |u_jj| (zeros above j); out[1]: two columns of workspace.
 // s_gam[j] is the gamma of u_j 2^{-s_ex[j]}.  Squares of the columns as they are
 // (s_ex = 0) serve while they stay inside FP64's range.  Where one of a panel's steps
 // met one outside (gamma is left at zero) the first form returns true and writes
@@ -376,9 +375,6 @@ __device__ __noinline__ bool panel_factor(double* W, const int* s_rem, const int
   const long long ub = __double_as_longlong(u), top = 0x7ffll << 52;
   const double mant = __longlong_as_double((ub & ~top) | (1023ll << 52));
   const double mu = copysign(recip_newton(fabs(mant)), mant);
-  const double b1 = on ? fabs(beta) : 1.0, zb = recip_newton(b1);
-  double tau = fabs(uj) * zb;
-  tau = fma(fma(-tau, b1, fabs(uj)), zb, tau);
 #pragma unroll
   for (int k = 0; k < KR; ++k) {
     const int r = l8 + LPC * k;
@@ -390,11 +386,6 @@ __device__ __noinline__ bool panel_factor(double* W, const int* s_rem, const int
                   : 0.0;
       if (own && r <= pc && r < m) col[r] = r == pc ? (WIDE ? beta * up : beta) : x[k];
     }
-  }
-  __syncwarp();
-  if (l8 == 0) {
-    s_beta[pc] = on ? tau : 0.0;
-    s_ex[pc] = (int)((ub & top) >> 52) - 1023;
   }
   return false;
 }
@@ -627,7 +618,7 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   int* s_rem = reinterpret_cast<int*>(s_key + N);              // [m]
   int* s_cand = s_rem + N;                                     // [CN] positions in rem
   int* s_sel = s_cand + CN;                                    // [32] candidate numbers
-  int* s_ex = s_sel + NB;                                      // [32] E_j (panel_factor)
+  int* s_ex = s_sel + NB;                                      // [32] exponents of gamma's vectors
   int* s_f0 = s_ex + NB;                                       // [32] the first set's s_f
   int* s_f = s_f0 + NB;                                        // [32] exponents of V^T's rows
   int* s_h = s_f + NB;                                         // [32] of V's columns times 2^{-rho_r}
@@ -760,8 +751,6 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   }
 #undef DQMC_FACTOR
   __syncthreads();
-  double* s_tau = s_beta;                   // (panel_factor's last step)
-  int* s_E = s_ex;
   uint32_t nm = 0;                          // MMA groups waited for
   for (int set = 0; set < a.sets; ++set) {
     // ---- exponents: first set of the columns alone, second set with the row scales and
@@ -803,7 +792,7 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
       s_er[tid] = mx == 0 ? 0 : mx - 100000 - 1020;
       a.er(z, p, 1)[j0 + tid] = s_er[tid];
     }
-    __syncthreads();
+    if (set) __syncthreads();
     // ---- digits of V^T (to the tiles and the staging ring) and V^T V: four 32-row
     // blocks at a time, in the second set two with their own left operands ------------
     {
@@ -867,8 +856,13 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
       gm[i * TLD + c] = stacked_value(ex, i, c, set ? s_h[i] + s_f[c] - s_f0[i] - s_f0[c] : 0);
     }
     double* s_g = xs;                       // (xs is free) tau_j 2^{2 (f_j - E_j)}
-    if (!set && tid < NB)
-      s_g[tid] = s_f[tid] < TC_NONFINITE / 2 ? scalbn(s_tau[tid], 2 * (s_f[tid] - s_E[tid])) : 0.0;
+    if (!set && tid < NB) {                 // tau_j = -u_jj / beta_j, a quotient in (1, 2]
+      const bool on = tid < nb && s_gam[tid] > 0.0 && s_f[tid] < TC_NONFINITE / 2;
+      const double b1 = on ? fabs(s_beta[tid]) : 1.0, n = on ? fabs(s_uj[tid]) : 0.0;
+      const double zb = recip_newton(b1), q = n * zb;
+      const int E = (int)((__double_as_longlong(us[tid * LDU + tid]) >> 52) & 0x7ff) - 1023;
+      s_g[tid] = scalbn(fma(fma(-q, b1, n), zb, q), on ? 2 * (s_f[tid] - E) : 0);
+    }
     for (int e = tid; e < NB * TLD; e += 512) tm[e] = 0.0;
     __syncthreads();
     // ---- T: T_jj = tau_j, T(:j, j) = -tau_j T(:j,:j) G(:j, j); 8 x 8 blocks by one
