@@ -149,3 +149,25 @@ def test_full_device_keeps_the_workspace(dq, graphs):
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("prec", [0, 8])
+@pytest.mark.parametrize("call", ["greens", "displaced", "gradient"])
+@pytest.mark.parametrize("N", [64, 160])
+def test_no_room_means_the_fp64_pipe(dq, N, call, prec):
+    """Under a limit that leaves no room for the digits no tensor-core kernel runs, and
+    without the limit they do: the fallback is what ran."""
+    K, V = _dev(di.chain_hopping(N)), _fields(9900 + N, 3, 8, N)
+    run = {"greens": dq.greens, "displaced": dq.greens_tdisplaced, "gradient": dq.logdet_grad}[call]
+    names = ("tc_gemm_kernel", "chain_tc_kernel", "qr_panel_kernel", "qr_apply_kernel", "solve_back_kernel")
+    free = dq.Handle(fold=0, chain_precision=prec)
+    ref = run(K, 0.1, V, 4, handle=free)
+    with_room = _kernels(lambda: run(K, 0.1, V, 4, handle=free))
+    assert any(n in k for k in with_room for n in names)
+    h = dq.Handle(fold=0, chain_precision=prec)
+    # one digit operand of one instance (8 planes of N padded to 128 by 32) too little
+    h.set_memory_limit(free.device_bytes * 8 // 9 - 16 * ((N + 127) // 128 * 128) * ((N + 31) // 32 * 32))
+    without = _kernels(lambda: run(K, 0.1, V, 4, handle=h))
+    assert not any(n in k for k in without for n in names)
+    out = run(K, 0.1, V, 4, handle=h)
+    assert (out[0] - ref[0]).abs().max().item() <= 1e-9 * max(1.0, ref[0].abs().max().item())
