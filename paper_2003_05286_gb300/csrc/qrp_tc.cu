@@ -31,20 +31,20 @@
 // Measured against the one-CTA kernels, whole factorisation, random graded
 // columns: N = 64 0.476 -> 0.265 ms (one instance) and 0.479 -> 0.301 (128), N =
 // 100 1.03 -> 0.55 and 1.03 -> 0.77, N = 256 7.76 -> 1.64 and 7.85 -> 2.95, N =
-// 324 22.6 -> 2.39 and 25.4 -> 5.40; same pivots, residuals no larger.  What is
+// 324 22.6 -> 2.37 and 25.4 -> 7.67; same pivots, residuals no larger.  What is
 // left at N = 256 (thousand cycles per panel of 256 rows): pivot search 140, FP64
 // panel 255 (the FP64 pipe, plus a square root, a division and two barriers per
 // column), digits and V^T V 27, T 12; an apply of 256 rows 55.
 //
-// V's columns are v_j = u_j / u_jj, H_j = 1 - tau_j v_j v_j^T with tau_j = (beta_j -
-// alpha_j) / beta_j.  A column that is a multiple of a unit vector then gives exact
-// digits, T and Q, and decoupled sites stay decoupled.  (With u_j scaled by powers of two
-// alone the rounding of gamma put 2^-53 into Q's zeros, times the grading of the next
-// chunk: K = 0, fields of variance 4, N = 160, M = 40, k = 10, error of G 6e-8 -> 1e-15;
-// one N = 256 factorisation 1.618 -> 1.626 ms.)  |v_r| <= 1 = v_j, so V needs no
-// exponents and T takes up the scales: every product is then accurate
-// column by column against the column's largest entry, as Householder's method
-// is.  When the rows of A are graded too (Drow: the levels of the tree fold, whose
+// V's columns are scaled by powers of two into (-1/4, 1/4) (|u_r| <= |u_j|), so
+// V needs no exponents and T takes up the scales.  A column whose entries differ by many
+// orders (or has zeros) is divided by its leading entry first: H_j = 1 - tau_j v_j v_j^T,
+// v_j = u_j / u_jj, tau_j = (beta_j - alpha_j) / beta_j, which are exact for a multiple of a
+// unit vector, as are its digits, T and Q, and decoupled sites stay decoupled.  (The
+// rounding of gamma put 2^-53 into Q's zeros, times the grading of the next chunk: K = 0,
+// fields of variance 4, N = 160, M = 40, k = 10, error of G 6e-8 -> 1e-15.)  Every
+// product is then accurate column by column against the column's largest entry, as
+// Householder's method is.  When the rows of A are graded too (Drow: the levels of the tree fold, whose
 // factor D_2 sits on the left), Householder QR with column pivoting is accurate
 // row by row (Cox and Higham, 1998), and so must be the update of A: it then uses
 // a second set of digits in which u_rj has the size s_r of row r: V W2 has row
@@ -70,6 +70,11 @@ constexpr int VT_TILE = 8 * DT;           // V^T: 8 digits x 32 panel columns x 
 constexpr int V_TILE = 8 * 128 * 64;      // V: 8 digits x 128 rows x 32 panel columns
 constexpr int RING = 4 * VT_TILE;         // staging of both kernels (64 KB)
 constexpr int TLD = 33;
+// Columns whose entries span more than 2^UNIT_SPAN get reflectors with leading entry one
+// (the head of this file).  A zero has exponent 0; a dense column of 256 random entries
+// spans some 2^12 and gains nothing, while the division, one multiplication an entry on the
+// FP64 pipe, takes up to 1% of an N = 256 factorisation (1.618 -> 1.631 ms with all columns).
+constexpr int UNIT_SPAN = 30;
 constexpr int QF = 2 * 8 * 52;             // floats of two staged FP32 columns (8 x 52 >= 4 x 68)
 constexpr int XS = QRTC_MAX_N;            // rows of a staged FP64 column
 enum { QP_SMALL, QP_MID, QP_BIG };        // forms of the panel kernel
@@ -273,8 +278,9 @@ __device__ __noinline__ void pivot_search(const double* W, const double* Din, co
 // holds its sub-partition's pipe for 64 cycles: short panels take 8 lanes (few
 // reduction levels, few warps), tall ones 16 (the columns left spread evenly
 // over the sub-partitions; N = 256, 32 columns: 323 -> 240 thousand cycles).  A
-// warp whose columns are done drops out.  Leaves R in W^T and in out[0] v_j 2^{E_j}, v_j =
-// u_j / u_jj, 2^{E_j} <= |u_jj| (zeros above j); out[1]: two columns of workspace.
+// warp whose columns are done drops out.  Leaves R in W^T and in out[0] (zeros above j)
+// u_j, or where s_unit[j] is set v_j 2^{E_j}, v_j = u_j / u_jj, 2^{E_j} <= |u_jj| < 2^{E_j + 1};
+// out[1]: two columns of workspace.
 // s_gam[j] is the gamma of u_j 2^{-s_ex[j]}.  Squares of the columns as they are
 // (s_ex = 0) serve while they stay inside FP64's range.  Where one of a panel's steps
 // met one outside (gamma is left at zero) the first form returns true and writes
@@ -284,7 +290,8 @@ __device__ __noinline__ void pivot_search(const double* W, const double* Din, co
 template <int LPC, int KR, bool SMALL, bool WIDE>
 __device__ __noinline__ bool panel_factor(double* W, const int* s_rem, const int* s_sel, int N,
                                           int j0, int m, int nb, int LDU, double* const* out,
-                                          double* s_beta, double* s_gam, double* s_uj, int* s_ex) {
+                                          double* s_beta, double* s_gam, double* s_uj, int* s_ex,
+                                          int* s_unit) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned FULL = 0xffffffffu;
   constexpr int CPW = 32 / LPC;             // columns per warp
@@ -368,25 +375,39 @@ __device__ __noinline__ bool panel_factor(double* W, const int* s_rem, const int
   }
   // (written before the last barrier of the loop: every warp sees the same)
   if (!WIDE && __any_sync(FULL, lane < nb && s_gam[lane] == 0.0)) return true;
-  // u_j is left as v_j 2^{E_j}: the leading entry, and one as large, exactly +-2^{E_j}
   const double up = WIDE && own ? scalbn(1.0, s_ex[pc]) : 1.0;
   const bool on = own && s_gam[pc] > 0.0;
   const double beta = own ? s_beta[pc] : 0.0, uj = on ? s_uj[pc] : 1.0, u = WIDE ? uj * up : uj;
   const long long ub = __double_as_longlong(u), top = 0x7ffll << 52;
-  const double mant = __longlong_as_double((ub & ~top) | (1023ll << 52));
-  const double mu = copysign(recip_newton(fabs(mant)), mant);
+  int least = 0x7ff;                       // exponent of the smallest entry below the leading one
+#pragma unroll
+  for (int k = 0; k < KR; ++k) {
+    const int r = l8 + LPC * k;
+    if (r > pc && r < m) least = min(least, (int)((__double_as_longlong(x[k]) >> 52) & 0x7ff));
+  }
+#pragma unroll
+  for (int o = 1; o < LPC; o <<= 1) least = min(least, __shfl_xor_sync(FULL, least, o));
+  const bool unit = on && least < (int)((ub & top) >> 52) - UNIT_SPAN;
+  const bool some = __any_sync(FULL, unit);
+  double mu = 1.0;
+  if (some && unit) {
+    const double mant = __longlong_as_double((ub & ~top) | (1023ll << 52));
+    mu = copysign(recip_newton(fabs(mant)), mant);
+  }
 #pragma unroll
   for (int k = 0; k < KR; ++k) {
     const int r = l8 + LPC * k;
     if (r < rows) {
-      const double xr = r == pc ? u : x[k];
-      const long long xb = __double_as_longlong(xr) ^ ub;
-      us[r] = on && r < m && r >= pc
-                  ? ((xb << 1) == 0 ? __longlong_as_double((ub & top) | (xb & (1ll << 63))) : xr * mu)
-                  : 0.0;
+      double v = r == pc ? u : x[k];
+      if (some) {                          // the leading entry, and one as large, exactly +-2^{E_j}
+        const long long xb = __double_as_longlong(v) ^ ub;
+        v = unit && (xb << 1) == 0 ? __longlong_as_double((ub & top) | (xb & (1ll << 63))) : v * mu;
+      }
+      us[r] = on && r < m && r >= pc ? v : 0.0;
       if (own && r <= pc && r < m) col[r] = r == pc ? (WIDE ? beta * up : beta) : x[k];
     }
   }
+  if (l8 == 0) s_unit[pc] = unit;
   return false;
 }
 
@@ -619,7 +640,8 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
   int* s_cand = s_rem + N;                                     // [CN] positions in rem
   int* s_sel = s_cand + CN;                                    // [32] candidate numbers
   int* s_ex = s_sel + NB;                                      // [32] exponents of gamma's vectors
-  int* s_f0 = s_ex + NB;                                       // [32] the first set's s_f
+  int* s_unit = s_ex + NB;                                     // [32] columns with leading entry one
+  int* s_f0 = s_unit + NB;                                       // [32] the first set's s_f
   int* s_f = s_f0 + NB;                                        // [32] exponents of V^T's rows
   int* s_h = s_f + NB;                                         // [32] of V's columns times 2^{-rho_r}
   int* s_rho = s_h + NB;                                       // [32 nkl]
@@ -728,11 +750,11 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
     bool redo = false;                                                                            \
     if (wid < LPC_)                                                                               \
       redo = panel_factor<LPC_, KR_, SIZE == QP_SMALL, false>(W, s_rem, s_sel, N, j0, m, nb, LDU, \
-                                                              out, s_beta, s_gam, s_uj, s_ex);    \
+                                                              out, s_beta, s_gam, s_uj, s_ex, s_unit); \
     if (redo) {                             /* (alike in these warps) */                          \
       asm volatile("bar.sync 1, %0;" ::"n"(32 * LPC_) : "memory");                                \
       panel_factor<LPC_, KR_, SIZE == QP_SMALL, true>(W, s_rem, s_sel, N, j0, m, nb, LDU, out,    \
-                                                      s_beta, s_gam, s_uj, s_ex);                 \
+                                                      s_beta, s_gam, s_uj, s_ex, s_unit);         \
     }                                                                                             \
   } while (0)
   {
@@ -855,17 +877,20 @@ __global__ void __launch_bounds__(512, SIZE == QP_SMALL ? 2 : 1) qr_panel_kernel
       const int i = e & 31, c = e >> 5;
       gm[i * TLD + c] = stacked_value(ex, i, c, set ? s_h[i] + s_f[c] - s_f0[i] - s_f0[c] : 0);
     }
-    double* s_g = xs;                       // (xs is free) tau_j 2^{2 (f_j - E_j)}
-    if (!set && tid < NB) {                 // tau_j = -u_jj / beta_j, a quotient in (1, 2]
-      const bool on = tid < nb && s_gam[tid] > 0.0 && s_f[tid] < TC_NONFINITE / 2;
-      const double b1 = on ? fabs(s_beta[tid]) : 1.0, n = on ? fabs(s_uj[tid]) : 0.0;
-      const double zb = recip_newton(b1), q = n * zb;
-      const int E = (int)((__double_as_longlong(us[tid * LDU + tid]) >> 52) & 0x7ff) - 1023;
-      s_g[tid] = scalbn(fma(fma(-q, b1, n), zb, q), on ? 2 * (s_f[tid] - E) : 0);
+    double* s_g = xs;                       // (xs is free) gamma of u_j 2^{-f_j}, tau_j of v_j 2^{E_j - f_j}
+    if (!set && tid < NB) {
+      double g = tid < nb && s_f[tid] < TC_NONFINITE / 2 ? s_gam[tid] : 0.0;
+      int e = s_ex[tid];
+      if (g > 0.0 && s_unit[tid]) {         // tau_j = -u_jj / beta_j, a quotient in (1, 2]
+        const double b1 = fabs(s_beta[tid]), zb = recip_newton(b1), n = fabs(s_uj[tid]), q = n * zb;
+        g = fma(fma(-q, b1, n), zb, q);
+        e = (int)((__double_as_longlong(us[tid * LDU + tid]) >> 52) & 0x7ff) - 1023;
+      }
+      s_g[tid] = scalbn(g, 2 * (s_f[tid] - e));
     }
     for (int e = tid; e < NB * TLD; e += 512) tm[e] = 0.0;
     __syncthreads();
-    // ---- T: T_jj = tau_j, T(:j, j) = -tau_j T(:j,:j) G(:j, j); 8 x 8 blocks by one
+    // ---- T: T_jj = gamma_j, T(:j, j) = -gamma_j T(:j,:j) G(:j, j); 8 x 8 blocks by one
     // warp each, then T12 = -T11 (G12 T22) twice ---------------------------------------
     if (wid < 4 && lane < 8) {
       const int o = 8 * wid;
@@ -1233,7 +1258,7 @@ size_t apply_smem(int nkb) {
 }
 size_t panel_smem(int N, int nkb, bool small = false) {
   return 1024 + RING + ((size_t)NB * (32 * nkb + 1) + 2 * NB * TLD + 2 * xs_rows(small) + 3 * NB) * 8 +
-         (3 * QF + 2 + 2 * N + 128 + 5 * NB + 64 * nkb + 32) * 4 + 64;
+         (3 * QF + 2 + 2 * N + 128 + 6 * NB + 64 * nkb + 32) * 4 + 64;
 }
 }  // namespace
 
