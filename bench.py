@@ -663,6 +663,8 @@ def run_gpu(args, wl, rank, world):
         m_bad = int((stm != 0).sum().item())
         mixed = {"value": job_value(batch, world, args.steps, mms), "unit": "G/s",
                  "ms_per_step": mms / args.steps, "chain_precision": f"bf16x{args.mixed_slices}",
+                 **({"note": "DQMC_CHAIN_BF16X8 runs the FP64 chain's kernels"}
+                    if args.mixed_slices == 8 else {}),
                  "speedup_vs_fp64": tot_ms / mms,
                  "status_nonzero": m_bad,
                  "max_abs_dG_vs_fp64_path": float((Gm - G64).abs().max().item()),
@@ -768,7 +770,7 @@ def run_gpu(args, wl, rank, world):
         "metric": "greens_functions_per_second", "value": value, "unit": "G/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": tot_ms / args.steps, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f64" if prec == 0 else f"bf16x{prec}+f64", "data": "synthetic",
+        "vs_baseline": None, "dtype": "f64" if prec in (0, 8) else f"bf16x{prec}+f64", "data": "synthetic",
         "config": {"workload": args.workload, "N": N, "M": M, "k": k, "beta": wl["beta"],
                    "U": wl["U"], "dtau": wl["dtau"], "instances_per_gpu": batch,
                    "chain_precision": args.precision, "cuda_graphs": graphs, "fold": args.fold,
@@ -943,7 +945,7 @@ def measure_other(args, wl, rank, world, peak=None):
     line = {"metric": metric, "value": job_value(batch, world, args.steps, tot), "unit": unit,
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": tot / args.steps, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "f64" if prec == 0 else f"bf16x{prec}+f64",
+            "vs_baseline": None, "dtype": "f64" if prec in (0, 8) else f"bf16x{prec}+f64",
             "data": "synthetic",
             "config": dict(workload=name, baseline_config=wl["config"], instances_per_gpu=batch,
                            chain_precision=prec, cuda_graphs=graphs, fold=args.fold,

@@ -79,7 +79,10 @@ enum dqmc_status_bits {
  * tensor cores and are recombined in FP64; a product is accurate to about
  * N 2^{-7s-1} of (row max x column max), normwise rather than elementwise.
  * The FP64 products themselves run on the tensor cores from N = 33 (eight
- * base-256 digits, about N 2^{-58}), and DQMC_CHAIN_BF16X8 uses the FP64 chain.
+ * base-256 digits, at most N 2^{-57} of row max x column max: below FP64 FMAs
+ * normwise, not entry by entry, so that strong fields on weakly coupled sites
+ * lose more places than they do on the FP64 pipe), and DQMC_CHAIN_BF16X8 uses
+ * the FP64 chain.
  * Supported for N <= 256 in dqmc_greens, dqmc_logdet, dqmc_greens_tdisplaced,
  * dqmc_logdet_grad (both stacks) and dqmc_greens_ragged (every instance N <= 256);
  * N > 256 returns DQMC_ERR_UNSUPPORTED (dqmc_greens_noalloc takes no handle
@@ -164,6 +167,9 @@ dqmc_status dqmc_set_inversion_scheme(dqmc_handle h, int scheme);
 /* Decomposition that stabilises the chains (Sec. 4.2):
  *   DQMC_DECOMP_QR      (default) column-pivoted Householder QR, U D X with X
  *                       triangular up to the pivot permutation (Sec. 4.2.2);
+ *                       from N = 129 to 384 the pivots of each 32-column panel
+ *                       are taken among the 128 (N > 256: 64) columns of
+ *                       largest norm at its start;
  *   DQMC_DECOMP_JACOBI  one-sided Jacobi SVD, U D V^T with X = V^T orthogonal
  *                       (the accurate SVD variant of Sec. 4.2.1); about ten
  *                       sweeps of N^2/2 plane rotations each, so 10-50x the

@@ -185,8 +185,8 @@ cudaError_t lu_solve_f64(const LuArgs& a, cudaStream_t st);
 // 160, by N alone so that an instance's result does not depend on its batch; N
 // right-hand sides, LU -> QR: N = 144 1.76 -> 0.70 ms (1 instance), 1.81 -> 1.62
 // (128), 10.4 -> 13.8 (1024); N = 200 3.81 -> 1.05 and 3.93 -> 2.94 (128); N = 256
-// 6.92 -> 1.28 and 8.30 -> 3.99; N = 324 14.8 -> 2.02 and 19.5 -> 8.08; residuals
-// a fifth of the LU's.
+// 6.92 -> 1.26 and 8.30 -> 3.94; N = 324 14.8 -> 1.99 and 19.5 -> 9.49 (two passes of
+// 64: 512 MB hold 100 slots); residuals a fifth of the LU's.
 constexpr int SOLVETC_MIN_N = 160;
 size_t solve_tc_slot_bytes(int N);
 cudaError_t solve_tc(const LuArgs& a, void* ws, int slots, cudaStream_t st);

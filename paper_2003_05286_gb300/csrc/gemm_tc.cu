@@ -15,10 +15,11 @@
 //     K (pairs in the group) 2^14 <= 2^24: groups 0..3 (at most 4 pairs) may
 //     sum over 256 values of k, groups 4..7 over 128, after which they are
 //     drained into 64-bit integers and start again from zero;
-//   * pairs with p + q >= 8 are dropped: seven weights of 2^{-80} whose sum is
-//     below K 7 2^{-66} in scaled units, that is K 2^{-58} of
-//     (row max x column max) at worst and sqrt(K) 2^{-63} for digits of random
-//     sign, against K 2^{-53} and sqrt(K) 2^{-54} for K FP64 FMAs;
+//   * pairs with p + q >= 8 are dropped: 7.03 2^{-66} a term at most in scaled
+//     units, with the rounding of both operands 8.03 2^{-66}.  The maxima of row
+//     and column are at least 1/8 there: K 2^{-57} of (row max x column max) at
+//     worst and some sqrt(K) 2^{-62} for digits of random sign, against K 2^{-53}
+//     and sqrt(K) 2^{-54} for K FP64 FMAs (tests/test_gpu_digit_arithmetic.py);
 //   * the epilogue adds the groups exactly in integers and rounds once to FP64.
 // So the result is at least as accurate as the FMA chain normwise (against
 // row max x column max); entries far below their row's and column's largest

@@ -73,7 +73,7 @@ __host__ __device__ constexpr uint32_t oz_idesc(int n) {
 
 }  // namespace
 
-// Pair table: up to 36 (p, q) digit pairs (s <= 8) with their accumulator group.
+// Pair table: up to 28 (p, q) digit pairs (s <= 7) with their accumulator group.
 struct OzPairs {
   int n;                 // number of pairs
   int ngroups;           // accumulators (<= 8)
